@@ -320,12 +320,23 @@ __global__ void __launch_bounds__(kMeanThreads) k_field_sums(const DomainConst P
   if (threadIdx.x < 2) partials[2 * blockIdx.x + threadIdx.x] = sh[threadIdx.x][0];
 }
 
-__global__ void k_field_sums_final(const double* __restrict__ partials, int nblocks,
-                                   double* __restrict__ sums) {
-  if (threadIdx.x >= 2) return;
+// Adds the block sums in a fixed tree. One block, latency-bound: a single thread per sum
+// walking the 1216 partials took 84-94 us (a dependent load and FP64 addition each); with
+// 256 threads and a shared-memory tree a start from caller fields is 70-80 us shorter.
+__global__ void __launch_bounds__(kMeanThreads) k_field_sums_final(const double* __restrict__ partials,
+                                                                   int nblocks,
+                                                                   double* __restrict__ sums) {
+  __shared__ double sh[2][kMeanThreads];
+  const int j = threadIdx.x & 1;  // neighbouring threads take the two sums of one block
   double r = 0.0;
-  for (int b = 0; b < nblocks; ++b) r += partials[2 * b + threadIdx.x];
-  sums[threadIdx.x] = r;
+  for (int b = threadIdx.x >> 1; b < nblocks; b += kMeanThreads / 2) r += partials[2 * b + j];
+  sh[j][threadIdx.x >> 1] = r;
+  __syncthreads();
+  for (int half = kMeanThreads / 4; half > 0; half >>= 1) {
+    if ((int)(threadIdx.x >> 1) < half) sh[j][threadIdx.x >> 1] += sh[j][(threadIdx.x >> 1) + half];
+    __syncthreads();
+  }
+  if (threadIdx.x < 2) sums[threadIdx.x] = sh[threadIdx.x][0];
 }
 
 int grid_for(long long n, int block) {
@@ -429,9 +440,14 @@ cudaError_t launch_field_means(const DomainConst& P, const InitSpec& spec, doubl
                                cudaStream_t s) {
   // sums holds 2 results followed by 2 * kMeanBlocks partials
   double* partials = sums + 2;
-  k_field_sums<<<kMeanBlocks, kMeanThreads, 0, s>>>(P, spec, field_sample(P.ncell).run_stride,
-                                                     partials);
-  k_field_sums_final<<<1, 32, 0, s>>>(partials, kMeanBlocks, sums);
+  const long long stride = field_sample(P.ncell).run_stride;
+  // no more blocks than the sample fills: one block of a thread per cell each (the sums
+  // are the same; with all of them small domains paid for 1216 empty trees, 12 us)
+  const long long runs = (P.ncell + kTile - 1) / kTile, sampled = (runs + stride - 1) / stride;
+  long long blocks = (sampled * kTile + kMeanThreads - 1) / kMeanThreads;
+  if (blocks > kMeanBlocks) blocks = kMeanBlocks;
+  k_field_sums<<<(unsigned)blocks, kMeanThreads, 0, s>>>(P, spec, stride, partials);
+  k_field_sums_final<<<1, kMeanThreads, 0, s>>>(partials, (int)blocks, sums);
   return cudaGetLastError();
 }
 
