@@ -7,8 +7,10 @@
 // kernel's diagnostic variant fills the same field and writes one record per warp
 // instead (step_diag.cuh), which pass R folds into per-block records. Pass B takes
 // central differences of u from the field. Each pass writes one record per block
-// (warp shuffles, then shared memory) and a single block reduces the records in a
-// fixed order, so results are reproducible run to run.
+// (warp shuffles, then shared memory) and the last block of pass B to finish reduces the
+// records in a fixed order, so results are reproducible run to run.
+#include <atomic>
+
 #include "diag_device.cuh"
 #include "lbm_internal.h"
 
@@ -41,7 +43,9 @@ template <typename S, int PARITY, bool HELD>
 __global__ void __launch_bounds__(kBlock) k_diag_a(const DomainConst P, const S* __restrict__ pop,
                                                    const float* __restrict__ ghost,
                                                    float* __restrict__ ufield,
-                                                   double* __restrict__ partials) {
+                                                   double* __restrict__ partials,
+                                                   unsigned* __restrict__ ticket) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;  // pass B counts its blocks with it
   DiagAcc acc;
   diag_zero(acc);
   const long long n = P.ncell;
@@ -68,7 +72,9 @@ __global__ void __launch_bounds__(kBlock) k_diag_a(const DomainConst P, const S*
 // block (block b takes a contiguous range, in order).
 __global__ void __launch_bounds__(kBlock) k_diag_records(const float* __restrict__ rec,
                                                          long long nrec,
-                                                         double* __restrict__ partials) {
+                                                         double* __restrict__ partials,
+                                                         unsigned* __restrict__ ticket) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;
   const long long per = (nrec + gridDim.x - 1) / gridDim.x;
   const long long lo = blockIdx.x * per;
   const long long hi = lo + per < nrec ? lo + per : nrec;
@@ -101,7 +107,7 @@ __global__ void __launch_bounds__(kBlock) k_diag_records(const float* __restrict
 // addition. Every value of the field is read from DRAM about once (the halo comes
 // from L2: neighbouring columns are processed at about the same z).
 constexpr int kCells = 4;  // consecutive cells of a row per thread
-constexpr int kTileX = 32, kTileY = 16, kZChunk = 32, kRingB = 4;
+constexpr int kTileX = 32, kTileY = 16, kRingB = 4;
 constexpr int kThreadsX = kTileX / kCells, kBlockB = kThreadsX * kTileY;
 constexpr int kRowF = kTileX + 8;           // 3 pad, x - 1 halo, 32 cells, x + 32 halo, 3 pad
 constexpr int kRowsB = kTileY + 2;          // y - 1 halo, 16 rows, y + 16 halo
@@ -140,12 +146,61 @@ __device__ __forceinline__ void ldv(const float* p, float (&o)[kCells]) {
   }
 }
 
+// Fixed-order FP64 reduction of the block records of both passes by one block of
+// kBlockB threads: thread (j, s) folds records s, s + 8, ... of quantity j, then the 8
+// slices are added in order. The reference density and energy are added back once per
+// cell at the end, the maximum Mach number is the root of the maximum of Mach^2 and the
+// maximum CFL number the maximum speed / c. Latency-bound (a few hundred KB): as a kernel
+// of its own over a fixed 1216 records, with every thread holding all 15 quantities and
+// an FP64 tree over 256 threads, it took 20 us whatever the domain.
+__device__ void diag_final(const DomainConst& P, const double* __restrict__ pa, int nblocks_a,
+                           const double* __restrict__ pb, int nblocks_b, double* __restrict__ out) {
+  constexpr int kN = kDiagA + 2, kSlices = kBlockB / 16;
+  __shared__ double sh[kSlices][16];
+  const int j = threadIdx.x & 15, sl = threadIdx.x >> 4;
+  if (j < 9 || j >= kDiagA) {  // sums
+    double r = 0.0;
+    if (j < 9) {
+      for (int b = sl; b < nblocks_a; b += kSlices) r += __ldcg(pa + (long long)b * kDiagA + j);
+    } else if (j < kN) {
+      for (int b = sl; b < nblocks_b; b += kSlices) r += __ldcg(pb + (long long)b * 2 + (j - kDiagA));
+    }
+    sh[sl][j] = r;
+  } else {  // extrema: FP32 values held in FP64
+    const bool mx = j < 11;
+    float r = mx ? -INFINITY : INFINITY;
+    for (int b = sl; b < nblocks_a; b += kSlices) {
+      const float v = (float)__ldcg(pa + (long long)b * kDiagA + j);
+      r = mx ? fmaxf(r, v) : fminf(r, v);
+    }
+    sh[sl][j] = r;
+  }
+  __syncthreads();
+  if (threadIdx.x < kN) {
+    const bool sum = j < 9 || j >= kDiagA, mx = j < 11;
+    double v = sh[0][j];
+    for (int q = 1; q < kSlices; ++q) {
+      if (sum) v += sh[q][j];
+      else v = mx ? fmaxf((float)v, (float)sh[q][j]) : fminf((float)v, (float)sh[q][j]);
+    }
+    if (j == 0) v += (double)P.rho_ref * (double)P.ncell;
+    if (j == 4) v += (double)P.E_ref * (double)P.ncell;
+    if (j == 9) v = sqrt(v);
+    if (j == 10) v = v / (double)P.c;
+    out[j] = v;
+  }
+}
+
 // kVec: nx is a multiple of 32, so every tile row is a full, 16-byte aligned row of 32
 // cells (vector copies and loads); otherwise element copies with wrapped x.
 template <bool kVec>
 __global__ void __launch_bounds__(kBlockB, 4) k_diag_b(const DomainConst P,
                                                     const float* __restrict__ ufield,
-                                                    double* __restrict__ partials) {
+                                                    int zchunk,
+                                                    const double* __restrict__ pa, int nblocks_a,
+                                                    double* __restrict__ partials,
+                                                    unsigned* __restrict__ ticket,
+                                                    double* __restrict__ out) {
   extern __shared__ __align__(16) float ring[];  // [kRingB][3][kRowsB][kRowF]
   __shared__ long long rowoff[kRowsB];           // (wrapped y) * nx of each tile row
   __shared__ int halo_x[2];                      // wrapped x0 - 1 and x0 + 32
@@ -154,7 +209,7 @@ __global__ void __launch_bounds__(kBlockB, 4) k_diag_b(const DomainConst P,
   const float inv_2dx = (float)(0.5 / P.dx64);
   const float s2 = mul(inv_2dx, inv_2dx);
   const int cols_x = (P.nx + kTileX - 1) / kTileX, cols_y = (P.ny + kTileY - 1) / kTileY;
-  const int chunks = (P.nz + kZChunk - 1) / kZChunk;
+  const int chunks = (P.nz + zchunk - 1) / zchunk;
   const long long items = (long long)cols_x * cols_y * chunks;
   const long long nxy = (long long)P.nx * P.ny;
   const int tx = threadIdx.x % kThreadsX, ty = threadIdx.x / kThreadsX;  // cells kCells tx... of row ty
@@ -163,7 +218,7 @@ __global__ void __launch_bounds__(kBlockB, 4) k_diag_b(const DomainConst P,
     const long long r = it / cols_x;
     const int cy = (int)(r % cols_y), cz = (int)(r / cols_y);
     const int x0 = cx * kTileX, y0 = cy * kTileY;
-    const int z0 = cz * kZChunk, z1 = min(z0 + kZChunk, P.nz);
+    const int z0 = cz * zchunk, z1 = min(z0 + zchunk, P.nz);
     const int np = z1 - z0 + 2;  // planes z0 - 1 ... z1 (wrapped)
     constexpr bool vec = kVec;
     if (threadIdx.x < kRowsB) rowoff[threadIdx.x] = (long long)wrap_index(y0 - 1 + threadIdx.x, P.ny) * P.nx;
@@ -373,108 +428,115 @@ __global__ void __launch_bounds__(kBlockB, 4) k_diag_b(const DomainConst P,
     FF r = sh[0][threadIdx.x];
     for (int w = 1; w < kBlockB / 32; ++w) ff_merge(r, sh[w][threadIdx.x]);
     partials[(long long)blockIdx.x * 2 + threadIdx.x] = ff_value(r);
+    __threadfence();  // the record is visible before the ticket counts this block
+  }
+  // The block that takes the last ticket sees every block's record and finishes.
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (last) {
+    __threadfence();
+    diag_final(P, pa, nblocks_a, partials, gridDim.x, out);
   }
 }
 
 constexpr size_t kDiagBSmem = sizeof(float) * kRingB * kPlaneB;
 
-// Grid of pass B: the blocks resident on the device at once (one wave), at most
-// kDiagBlocks (the partials buffer holds that many).
+// Blocks of pass B resident on the current device at once (one wave), at most kDiagBlocks
+// (the partials buffer holds that many). A property of the device and the kernel, so it
+// is looked up once per device.
 template <bool kVec>
-int diag_b_grid() {
+int diag_b_resident() {
+  constexpr int kMaxDevices = 64;
+  static std::atomic<int> known[kMaxDevices];
   int dev = 0, sms = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return kDiagBlocks;
+  if (dev < kMaxDevices) {
+    const int g = known[dev].load(std::memory_order_relaxed);
+    if (g > 0) return g;
+  }
   if (cudaFuncSetAttribute(k_diag_b<kVec>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)kDiagBSmem) != cudaSuccess ||
-      cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_diag_b<kVec>, kBlockB, kDiagBSmem) !=
           cudaSuccess) {
     cudaGetLastError();
     return kDiagBlocks;
   }
-  const int g = sms * per_sm;
-  return g < 1 ? 1 : (g > kDiagBlocks ? kDiagBlocks : g);
-}
-
-// Pass B into pb; returns its grid (the number of records written).
-int launch_b(const DomainConst& P, const float* ufield, double* pb, cudaStream_t s) {
-  if (P.nx % kTileX == 0) {
-    const int g = diag_b_grid<true>();
-    k_diag_b<true><<<g, kBlockB, kDiagBSmem, s>>>(P, ufield, pb);
-    return g;
-  }
-  const int g = diag_b_grid<false>();
-  k_diag_b<false><<<g, kBlockB, kDiagBSmem, s>>>(P, ufield, pb);
+  int g = sms * per_sm;
+  g = g < 1 ? 1 : (g > kDiagBlocks ? kDiagBlocks : g);
+  if (dev < kMaxDevices) known[dev].store(g, std::memory_order_relaxed);
   return g;
 }
 
-// Fixed-order FP64 reduction of the block records of both passes (nblocks records of
-// pass A or R, nblocks_b <= nblocks of pass B; one block of kBlock threads): thread t
-// folds blocks t, t + kBlock, ... of every quantity, then a
-// shared-memory tree combines the threads in a fixed pattern. The reference density
-// and energy are added back once per cell at the end, the maximum Mach number is the
-// root of the maximum of Mach^2 and the maximum CFL number the maximum speed / c.
-__global__ void __launch_bounds__(kBlock) k_diag_final(const DomainConst P,
-                                                       const double* __restrict__ pa,
-                                                       const double* __restrict__ pb, int nblocks,
-                                                       int nblocks_b, double* __restrict__ out) {
-  constexpr int kN = kDiagA + 2;
-  __shared__ double sh[kN][kBlock];
-  const int t = threadIdx.x;
-  double r[kN];
-#pragma unroll
-  for (int j = 0; j < kN; ++j) r[j] = (j >= 9 && j < 11) ? -INFINITY : ((j == 11 || j == 12) ? INFINITY : 0.0);
-  for (int b = t; b < nblocks; b += kBlock) {
-#pragma unroll
-    for (int j = 0; j < kDiagA; ++j) {
-      const double v = pa[(long long)b * kDiagA + j];
-      r[j] = j < 9 ? r[j] + v : (j < 11 ? fmax(r[j], v) : fmin(r[j], v));
-    }
-    if (b < nblocks_b) {
-      r[kDiagA] += pb[(long long)b * 2];
-      r[kDiagA + 1] += pb[(long long)b * 2 + 1];
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < kN; ++j) sh[j][t] = r[j];
-  __syncthreads();
-  for (int half = kBlock / 2; half > 0; half >>= 1) {
-    if (t < half) {
-#pragma unroll
-      for (int j = 0; j < kN; ++j) {
-        const double v = sh[j][t + half];
-        sh[j][t] = (j < 9 || j >= kDiagA) ? sh[j][t] + v
-                                          : (j < 11 ? fmax(sh[j][t], v) : fmin(sh[j][t], v));
-      }
-    }
-    __syncthreads();
-  }
-  if (t < kN) {
-    double v = sh[t][0];
-    if (t == 0) v += (double)P.rho_ref * (double)P.ncell;
-    if (t == 4) v += (double)P.E_ref * (double)P.ncell;
-    if (t == 9) v = sqrt(v);
-    if (t == 10) v = v / (double)P.c;
-    out[t] = v;
-  }
+long long diag_b_columns(const DomainConst& P) {
+  return (long long)((P.nx + kTileX - 1) / kTileX) * ((P.ny + kTileY - 1) / kTileY);
 }
+
+// Planes per work item of pass B. A column of the whole height is one serial march, so
+// 64^3 has 8 of them for 608 resident blocks; cutting it costs two halo planes and about
+// two planes' time of set-up per piece. The number of planes that minimises rounds x
+// (planes + 4) is taken: 2 at 64^3, 4 at 128^3, 64 at 256^3. Even, so that the sums
+// over pairs of planes are the same for every cut.
+int diag_b_planes(const DomainConst& P, int resident) {
+  const long long cols = diag_b_columns(P);
+  int best = 2;
+  long long best_cost = -1;
+  for (int z = 2; z <= 128; z += 2) {
+    const long long items = cols * ((P.nz + z - 1) / z);
+    const long long cost = (items + resident - 1) / resident * ((z < P.nz ? z : P.nz) + 4);
+    if (best_cost < 0 || cost <= best_cost) {
+      best_cost = cost;
+      best = z;
+    }
+    if (z >= P.nz) break;
+  }
+  return best;
+}
+
+// Pass B, which also finishes the diagnostics (nblocks_a records of pass A or R in pa).
+template <bool kVec>
+void launch_b_t(const DomainConst& P, const float* ufield, const double* pa, int nblocks_a,
+                double* pb, unsigned* ticket, double* out, cudaStream_t s) {
+  const int resident = diag_b_resident<kVec>();
+  const int planes = diag_b_planes(P, resident);
+  const long long items = diag_b_columns(P) * ((P.nz + planes - 1) / planes);
+  const int g = items < resident ? (int)items : resident;
+  k_diag_b<kVec><<<g, kBlockB, kDiagBSmem, s>>>(P, ufield, planes, pa, nblocks_a, pb, ticket, out);
+}
+
+void launch_b(const DomainConst& P, const float* ufield, const double* pa, int nblocks_a, double* pb,
+              unsigned* ticket, double* out, cudaStream_t s) {
+  if (P.nx % kTileX == 0) launch_b_t<true>(P, ufield, pa, nblocks_a, pb, ticket, out, s);
+  else launch_b_t<false>(P, ufield, pa, nblocks_a, pb, ticket, out, s);
+}
+
+// Blocks of pass A or R for n cells or records: one per thread, at most kDiagBlocks.
+int blocks_for(long long n) {
+  const long long g = (n + kBlock - 1) / kBlock;
+  return g > kDiagBlocks ? kDiagBlocks : (int)g;
+}
+
+// The block counter of pass B: the last word of the 16 result doubles (15 are results).
+unsigned* ticket_of(double* out16) { return reinterpret_cast<unsigned*>(out16 + kDiagA + 2); }
 
 template <typename S, int PARITY, bool HELD>
 void launch_a(const DomainConst& P, const void* pop, const float* ghost, float* ufield, double* pa,
-              cudaStream_t s) {
-  k_diag_a<S, PARITY, HELD><<<kDiagBlocks, kBlock, 0, s>>>(P, static_cast<const S*>(pop), ghost,
-                                                           ufield, pa);
+              unsigned* ticket, cudaStream_t s) {
+  k_diag_a<S, PARITY, HELD><<<blocks_for(P.ncell), kBlock, 0, s>>>(P, static_cast<const S*>(pop), ghost,
+                                                                   ufield, pa, ticket);
 }
 
 template <typename S>
 void launch_a_store(const DomainConst& P, int parity, const void* pop, const float* ghost,
-                    float* ufield, double* pa, cudaStream_t s) {
+                    float* ufield, double* pa, unsigned* ticket, cudaStream_t s) {
   if (P.bc_x) {
-    if (parity) launch_a<S, 1, true>(P, pop, ghost, ufield, pa, s);
-    else launch_a<S, 0, true>(P, pop, ghost, ufield, pa, s);
+    if (parity) launch_a<S, 1, true>(P, pop, ghost, ufield, pa, ticket, s);
+    else launch_a<S, 0, true>(P, pop, ghost, ufield, pa, ticket, s);
   } else {
-    if (parity) launch_a<S, 1, false>(P, pop, ghost, ufield, pa, s);
-    else launch_a<S, 0, false>(P, pop, ghost, ufield, pa, s);
+    if (parity) launch_a<S, 1, false>(P, pop, ghost, ufield, pa, ticket, s);
+    else launch_a<S, 0, false>(P, pop, ghost, ufield, pa, ticket, s);
   }
 }
 
@@ -486,12 +548,11 @@ cudaError_t launch_diag(const DomainConst& P, int store, int parity, const void*
   double* pa = partials;
   double* pb = partials + (long long)kDiagBlocks * kDiagA;
   switch (store) {
-    case 0: launch_a_store<float>(P, parity, pop, ghost, ufield, pa, s); break;
-    case 1: launch_a_store<__half>(P, parity, pop, ghost, ufield, pa, s); break;
-    default: launch_a_store<__nv_bfloat16>(P, parity, pop, ghost, ufield, pa, s); break;
+    case 0: launch_a_store<float>(P, parity, pop, ghost, ufield, pa, ticket_of(out16), s); break;
+    case 1: launch_a_store<__half>(P, parity, pop, ghost, ufield, pa, ticket_of(out16), s); break;
+    default: launch_a_store<__nv_bfloat16>(P, parity, pop, ghost, ufield, pa, ticket_of(out16), s); break;
   }
-  const int gb = launch_b(P, ufield, pb, s);
-  k_diag_final<<<1, kBlock, 0, s>>>(P, pa, pb, kDiagBlocks, gb, out16);
+  launch_b(P, ufield, pa, blocks_for(P.ncell), pb, ticket_of(out16), out16, s);
   return cudaGetLastError();
 }
 
@@ -500,9 +561,9 @@ cudaError_t launch_diag_records(const DomainConst& P, const float* rec, long lon
                                 cudaStream_t s) {
   double* pa = partials;
   double* pb = partials + (long long)kDiagBlocks * kDiagA;
-  k_diag_records<<<kDiagBlocks, kBlock, 0, s>>>(rec, nrec, pa);
-  const int gb = launch_b(P, ufield, pb, s);
-  k_diag_final<<<1, kBlock, 0, s>>>(P, pa, pb, kDiagBlocks, gb, out16);
+  const int blocks = blocks_for(nrec);
+  k_diag_records<<<blocks, kBlock, 0, s>>>(rec, nrec, pa, ticket_of(out16));
+  launch_b(P, ufield, pa, blocks, pb, ticket_of(out16), out16, s);
   return cudaGetLastError();
 }
 

@@ -140,7 +140,8 @@ cudaError_t launch_plane(const DomainConst& P, int store, void* pop, int z, int 
 // Diagnostics (diag.cu).
 constexpr int kDiagA = 13;  // sums: rho mx my mz E ke nonfinite | max: mach cfl | min: rho T
 constexpr int kDiagBlocks = 1216;
-// ufield: 4 floats per cell of scratch; partials: kDiagBlocks * (kDiagA + 2) doubles.
+// ufield: 4 floats per cell of scratch; partials: kDiagBlocks * (kDiagA + 2) doubles;
+// out16: kDiagA + 2 results, and one word more as the block counter of the last pass.
 cudaError_t launch_diag(const DomainConst& P, int store, int parity, const void* pop,
                         const float* ghost, float* ufield, double* partials, double* out16,
                         cudaStream_t s);
