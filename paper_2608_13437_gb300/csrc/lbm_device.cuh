@@ -68,6 +68,46 @@ __device__ __forceinline__ bool lbm_check(const DomainConst& P, bool ok) {
 #define LBM_CHECK(P, cond) true
 #endif
 
+// ---------------------------------------------------------------- packed FP32 pairs
+// Two FP32 values in an aligned register pair and the packed operations of sm_100 and
+// later: each half is rounded exactly as the scalar operation with the same rounding, so
+// results are the scalar code's bit for bit at half the instructions. The cell update
+// works on pairs of neighbouring fields (k, k + 1), which the vector loads and stores of
+// the layout already hold in neighbouring registers.
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 pack2(float a, float b) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(F2 v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+  F2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// Only for products that no packed sum takes: a packed sum of a packed product was
+// contracted into one fused operation in some kernels and not in others, explicit
+// rounding or not (measured on 2^20 values); products that are summed are scalar, which
+// the explicit rounding does keep apart.
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 // ---------------------------------------------------------------- storage codecs
 // Scalar codecs (dec/enc) and the vector forms used by the step kernel: V4 holds
 // four consecutive fields of one direction of one cell, V2 two.
@@ -105,8 +145,8 @@ struct Codec16 {
   static __device__ __forceinline__ unsigned from_f2(float a, float b);
   static __device__ __forceinline__ void dec2w(unsigned w, const float* s, float* o) {
     const float2 f = to_f2(w);
-    o[0] = kScaled ? f.x * s[0] : f.x;
-    o[1] = kScaled ? f.y * s[1] : f.y;
+    o[0] = kScaled ? __fmul_rn(f.x, s[0]) : f.x;
+    o[1] = kScaled ? __fmul_rn(f.y, s[1]) : f.y;
   }
   static __device__ __forceinline__ void dec4(const V4& v, const float* s, float o[4]) {
     dec2w(v.x, s, o);
@@ -116,12 +156,20 @@ struct Codec16 {
     dec2w(v, s, o);
   }
   static __device__ __forceinline__ V4 enc4(const float i[4], const float* is) {
-    if (!kScaled) return make_uint2(from_f2(i[0], i[1]), from_f2(i[2], i[3]));
-    return make_uint2(from_f2(i[0] * is[0], i[1] * is[1]), from_f2(i[2] * is[2], i[3] * is[3]));
+    return make_uint2(enc2(i, is), enc2(i + 2, is + 2));
   }
-  static __device__ __forceinline__ V2 enc2(const float i[2], const float* is) {
-    if (!kScaled) return from_f2(i[0], i[1]);
-    return from_f2(i[0] * is[0], i[1] * is[1]);
+  static __device__ __forceinline__ void scaled(const float* i, const float* is, float& a, float& b) {
+    if (kScaled) {
+      unpack2(mul2(pack2(i[0], i[1]), pack2(is[0], is[1])), a, b);
+    } else {
+      a = i[0];
+      b = i[1];
+    }
+  }
+  static __device__ __forceinline__ V2 enc2(const float* i, const float* is) {
+    float a, b;
+    scaled(i, is, a, b);
+    return from_f2(a, b);
   }
   // Stochastic rounding of a pair (a to the low half, b to the high half): the
   // hardware conversion with random bits (cvt.rs, sm_100 and later) adds the low 16
@@ -132,21 +180,14 @@ struct Codec16 {
   static __device__ __forceinline__ unsigned from_f2_sr(float a, float b, unsigned r);
   static __device__ __forceinline__ V4 enc4_sr(const float i[4], const float* is, unsigned r0,
                                                unsigned r1) {
-    float a = i[0], b = i[1], c = i[2], e = i[3];
-    if (kScaled) {
-      a = a * is[0];
-      b = b * is[1];
-      c = c * is[2];
-      e = e * is[3];
-    }
+    float a, b, c, e;
+    scaled(i, is, a, b);
+    scaled(i + 2, is + 2, c, e);
     return make_uint2(from_f2_sr(a, b, r0), from_f2_sr(c, e, r1));
   }
   static __device__ __forceinline__ V2 enc2_sr(const float i[2], const float* is, unsigned r) {
-    float a = i[0], b = i[1];
-    if (kScaled) {
-      a = a * is[0];
-      b = b * is[1];
-    }
+    float a, b;
+    scaled(i, is, a, b);
     return from_f2_sr(a, b, r);
   }
 };
@@ -563,11 +604,11 @@ __device__ __forceinline__ float collide_cell(const DomainConst& P, float (&d)[k
   // Zeroth moments (Sec. 2.2: Q from the zeroth moment alone), i ascending.
   float D[kF];
 #pragma unroll
-  for (int k = 0; k < kF; ++k) {
-    float s = d[k][0];
+  for (int k = 0; k < kF; k += 2) {
+    F2 s = pack2(d[k][0], d[k + 1][0]);
 #pragma unroll
-    for (int i = 1; i < kQ; ++i) s = add(s, d[k][i]);
-    D[k] = s;
+    for (int i = 1; i < kQ; ++i) s = add2(s, pack2(d[k][i], d[k + 1][i]));
+    unpack2(s, D[k], D[k + 1]);
   }
   float Q[kF];
 #pragma unroll
@@ -626,27 +667,38 @@ __device__ __forceinline__ float collide_cell(const DomainConst& P, float (&d)[k
     so->omega_h = om;
     return D[0];
   } else {
-    // Collision, field by field: d* = d + omega_h (deq - d) + w_i dS_k with
-    // deq_0 = D/4, deq_{+-a} = D/8 +- Phi_a / (2c).
+    // Collision, by pairs of fields: d* = d + omega_h (deq - d) + w_i dS_k with
+    // deq_0 = D/4, deq_{+-a} = D/8 +- Phi_a / (2c). With the sums and updates in pairs the
+    // whole-tile-row step under the twist takes 738 instructions per warp instead of 910 in
+    // FP32 and 1071-1084 in FP16: no difference where HBM bounds it (512^3), 7 to 9 % where
+    // issue does (Sod 1024 x 4 x 4 4410 -> 4075 us, 64^3 FP16 series 4768 -> 4483 us).
+    const F2 om2 = pack2(om, om);
+    const float hic = P.half_inv_c;
 #pragma unroll
-    for (int k = 0; k < kF; ++k) {
-      float fx, fy, fz;
-      field_flux<float>(k, s, fx, fy, fz);
-      const float e0 = mul(0.25f, D[k]), e1 = mul(0.125f, D[k]);
-      const float ax = mul(P.half_inv_c, fx), ay = mul(P.half_inv_c, fy), az = mul(P.half_inv_c, fz);
-      d[k][0] = fma_(om, sub(e0, d[k][0]), d[k][0]);
-      d[k][1] = fma_(om, sub(add(e1, ax), d[k][1]), d[k][1]);
-      d[k][2] = fma_(om, sub(sub(e1, ax), d[k][2]), d[k][2]);
-      d[k][3] = fma_(om, sub(add(e1, ay), d[k][3]), d[k][3]);
-      d[k][4] = fma_(om, sub(sub(e1, ay), d[k][4]), d[k][4]);
-      d[k][5] = fma_(om, sub(add(e1, az), d[k][5]), d[k][5]);
-      d[k][6] = fma_(om, sub(sub(e1, az), d[k][6]), d[k][6]);
-      if (k >= 5) {  // the relaxation source of tau and q (zero for rho, rho u, E)
-        const float dS = mul(k < 11 ? P.src_R : P.src_q, D[k]);
-        const float s0 = mul(0.25f, dS), s1 = mul(0.125f, dS);
-        d[k][0] = add(d[k][0], s0);
+    for (int k = 0; k < kF; k += 2) {
+      float fx[2], fy[2], fz[2];
+      field_flux<float>(k, s, fx[0], fy[0], fz[0]);
+      field_flux<float>(k + 1, s, fx[1], fy[1], fz[1]);
+      const F2 e0 = pack2(mul(0.25f, D[k]), mul(0.25f, D[k + 1]));
+      const F2 e1 = pack2(mul(0.125f, D[k]), mul(0.125f, D[k + 1]));
+      const F2 flux[3] = {pack2(mul(hic, fx[0]), mul(hic, fx[1])), pack2(mul(hic, fy[0]), mul(hic, fy[1])),
+                          pack2(mul(hic, fz[0]), mul(hic, fz[1]))};
+      // the relaxation source of tau and q (zero for rho, rho u, E; field 4 shares its
+      // pair with 5 and adds -0, which leaves every value as it is)
+      F2 s0 = 0, s1 = 0;
+      if (k >= 4) {
+        const float a = mul(k < 11 ? P.src_R : P.src_q, D[k]);
+        const float b = mul(k + 1 < 11 ? P.src_R : P.src_q, D[k + 1]);
+        s0 = pack2(k == 4 ? -0.0f : mul(0.25f, a), mul(0.25f, b));
+        s1 = pack2(k == 4 ? -0.0f : mul(0.125f, a), mul(0.125f, b));
+      }
 #pragma unroll
-        for (int i = 1; i < kQ; ++i) d[k][i] = add(d[k][i], s1);
+      for (int i = 0; i < kQ; ++i) {
+        F2 v = pack2(d[k][i], d[k + 1][i]);
+        const F2 eq = i == 0 ? e0 : ((i & 1) ? add2(e1, flux[(i - 1) >> 1]) : sub2(e1, flux[(i - 1) >> 1]));
+        v = fma2(om2, sub2(eq, v), v);
+        if (k >= 4) v = add2(v, i == 0 ? s0 : s1);
+        unpack2(v, d[k][i], d[k + 1][i]);
       }
     }
     float probe = 0.0f;
