@@ -58,7 +58,9 @@ typedef enum {
   LBM_E_STATE = 5,      /* call not valid in the current state (e.g. step before init) */
   LBM_E_IO = 6,         /* checkpoint file could not be read or written, or is corrupt */
   LBM_E_TIMEOUT = 7     /* a bounded wait inside a kernel ran out (a staged step's wait for its
-                           own bulk copy): the state is incomplete; sticky until re-init */
+                           own bulk copy, or a block's wait for its neighbours where many
+                           steps of a small domain run in one launch): the state is
+                           incomplete; sticky until re-init */
 } lbm_status;
 
 /* Population storage. All arithmetic is FP32 in every mode.
@@ -189,7 +191,8 @@ size_t lbm_population_bytes(const lbm_params* p);
  * times, allocates the device state on the current CUDA device (LBM_E_NOMEM if it
  * does not fit) and returns an uninitialised handle in *out. The state is one
  * population buffer updated in place; nothing of size O(cells) is allocated
- * besides it until lbm_diag is first called. The handle is bound to that device
+ * besides it until lbm_diag is first called (small domains get exchange buffers of
+ * their bricks' surfaces, a few MB at most, for lbm_step's on-chip form). The handle is bound to that device
  * (lbm_info_t.device): every later call on it makes the device current while it
  * runs and restores the caller's current device before returning, so one thread can
  * drive handles on several GPUs. cuda_stream and pop_buffer must belong to it. */
@@ -248,7 +251,12 @@ lbm_status lbm_init_state(lbm_handle* h, const void* Q, int src_on_device, int d
  * steps; esoteric twist: own slots and one slot of each of the +x, +y, +z
  * neighbours on every step; lbm_params.streaming), computes moments, closure,
  * sensor and collision in FP32 and writes the 98 post-collision populations back
- * in place, so that streaming happens through the index maps. Asynchronous on the handle's stream. Returns LBM_E_STATE before
+ * in place, so that streaming happens through the index maps. With use_graphs, calls of
+ * 8 steps or more on small domains (up to about 58 thousand cells, where it is the faster
+ * form) run as one cooperative launch that keeps the populations on the chip between the
+ * steps; the result is the same bit for bit, and a wait between its blocks that runs out
+ * (bounded; it does not happen in normal operation) is reported as LBM_E_TIMEOUT.
+ * Asynchronous on the handle's stream. Returns LBM_E_STATE before
  * an init, LBM_E_NONFINITE if an earlier synchronising call saw non-finite
  * moments (no work is issued then). */
 lbm_status lbm_step(lbm_handle* h, int n);
@@ -344,7 +352,8 @@ lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out);
 
 /* Fixes the step kernel's form (variant 0-4, see lbm_info_t) and, for variants 0 and
  * 1, its block size (32, 64, 96 or 128 threads; ignored by the staged variants)
- * instead of the defaults or the autotuner's choice. The staged variants need a
+ * instead of the defaults or the autotuner's choice; small domains then take one launch
+ * per step too. The staged variants need a
  * periodic x axis, nx a multiple of 32 (whole 32-cell tiles per row), rounding to
  * nearest and the AA maps (streaming 0) (LBM_E_INVAL otherwise). All forms compute
  * bit-identical populations. A staged step whose wait

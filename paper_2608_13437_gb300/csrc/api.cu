@@ -173,7 +173,7 @@ struct lbm_handle {
   int block_x = 64;
   int variant = 0;             // step kernel: register budget (0, 1) or staged form (2-4)
   int staged_grid = 0;         // persistent grid of the staged forms
-  bool stalled = false;        // a staged step gave up waiting for a bulk copy
+  bool stalled = false;        // a step gave up a wait inside its kernel (flag bit 2)
   bool skip_next_copy = false; // test hook: the next direct staged step skips one copy
   cudaGraphExec_t g_pair = nullptr, g_chunk = nullptr;
   bool graphs_valid = false;
@@ -185,11 +185,20 @@ struct lbm_handle {
   double* hdiag = nullptr;     // pinned host copy of dout and the flag
   void* stage = nullptr;       // device staging for host-side outputs (kStageBytes)
   cudaEvent_t ev_diag = nullptr;
+  // resident form (step_resident.cu): bricks, their inboxes and step counts (one block)
+  ResidentPlan res;
+  bool res_on = false;         // the domain is small enough, and no kernel form was asked for
+  void* res_mem = nullptr;
+  size_t res_inbox = 0, res_bytes = 0;
 };
 
 namespace {
 
 constexpr int kChunkPairs = 16;  // a chunk graph holds 32 steps
+// The resident form is taken for calls of at least this many steps (a launch loads and
+// stores the whole state once); one launch of it takes at most kResidentMostSteps.
+constexpr int kResidentLeastSteps = 8;
+constexpr int kResidentMostSteps = 4096;
 
 #define LBM_CUDA(expr)                                                                        \
   do {                                                                                        \
@@ -220,7 +229,8 @@ cudaError_t step_launch(lbm_handle* h, int parity, cudaStream_t s) {
 }
 
 // Flag bits written by the step kernels: 1 = a non-finite moment, 2 = a staged step
-// gave up waiting for a bulk copy (its state is then incomplete).
+// gave up waiting for a bulk copy, or a block of the resident form for its neighbours
+// (the state is then incomplete).
 void latch_flag(lbm_handle* h, unsigned flag) {
   if (flag & 1u) h->nonfinite = true;
   if (flag & 2u) h->stalled = true;
@@ -255,6 +265,41 @@ lbm_status ensure_graphs(lbm_handle* h) {
   return LBM_OK;
 }
 
+// Sets up the resident form if the domain is small enough for the device. Its memory is a
+// fraction of the populations; without it the plain kernel serves.
+void setup_resident(lbm_handle* h) {
+  int sms = 0, coop = 0;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (!coop || !resident_plan(h->P, h->prm.store, sms, &h->res)) return;
+  h->res_inbox = resident_inbox_bytes(h->res, h->prm.store);
+  h->res_bytes = h->res_inbox + sizeof(unsigned) * (size_t)h->res.blocks();
+  if (cudaMalloc(&h->res_mem, h->res_bytes) != cudaSuccess ||
+      cudaMemset(h->res_mem, 0, h->res_bytes) != cudaSuccess ||
+      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+    cudaGetLastError();
+    if (h->res_mem) cudaFree(h->res_mem);
+    h->res_mem = nullptr;
+    return;
+  }
+  h->res_on = true;
+}
+
+// Whether the next n steps go through the resident form: not on a stream under capture,
+// where lbm_step answers as the graph replay does.
+bool use_resident(const lbm_handle* h, int n) {
+  if (!h->res_on || n < kResidentLeastSteps) return false;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st == cudaStreamCaptureStatusNone;
+}
+
 lbm_status direct_step(lbm_handle* h) {
   if (h->skip_next_copy && h->variant >= kFirstStagedVariant) {
     h->skip_next_copy = false;
@@ -286,6 +331,8 @@ void set_reference(lbm_handle* h, double rho_ref, double E_ref) {
 // Runs both init passes for an initial state: Q_ref must be set beforehand.
 lbm_status run_init(lbm_handle* h, InitSpec& sp) {
   reset_scales(h);
+  if (h->stalled && h->res_mem)  // blocks that gave up waiting left their step counts apart
+    LBM_CUDA(cudaMemsetAsync(h->res_mem, 0, h->res_bytes, h->stream));
   if (h->prm.store == LBM_STORE_F16) {
     LBM_CUDA(cudaMemsetAsync(h->maxbits, 0, kF * sizeof(unsigned), h->stream));
     LBM_CUDA(launch_init(h->P, h->prm.store, sp, 0, h->pop, h->ghost, h->maxbits, nullptr, h->stream));
@@ -415,6 +462,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_handle** out) {
   h->P.check = h->flag + 2;  // word 2 of the flag block: the checked build's address count
   if (cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking) != cudaSuccess)
     return cleanup(fail(LBM_E_CUDA, "cudaStreamCreate failed"));
+  if (p->use_graphs) setup_resident(h);
   *out = h;
   return LBM_OK;
 }
@@ -435,6 +483,7 @@ lbm_status lbm_destroy(lbm_handle* h) {
   if (h->dout) cudaFree(h->dout);
   if (h->wrec) cudaFree(h->wrec);
   if (h->stage) cudaFree(h->stage);
+  if (h->res_mem) cudaFree(h->res_mem);
   if (h->hdiag) cudaFreeHost(h->hdiag);
   if (h->ev_diag) cudaEventDestroy(h->ev_diag);
   if (h->cap) cudaStreamDestroy(h->cap);
@@ -577,7 +626,7 @@ lbm_status lbm_step(lbm_handle* h, int n) {
   if (n < 0) return fail(LBM_E_INVAL, "n must be >= 0");
   if (!h->initialized) return fail(LBM_E_STATE, "lbm_step before an init");
   if (h->nonfinite) return fail(LBM_E_NONFINITE, "non-finite moments were detected earlier");
-  if (h->stalled) return fail(LBM_E_TIMEOUT, "a staged step gave up waiting for a bulk copy; re-init");
+  if (h->stalled) return fail(LBM_E_TIMEOUT, "a step gave up waiting for a bulk copy or a neighbouring block; re-init");
   if (n == 0) return LBM_OK;
   if (!h->prm.use_graphs) {
     for (int j = 0; j < n; ++j) {
@@ -590,6 +639,16 @@ lbm_status lbm_step(lbm_handle* h, int n) {
     lbm_status s0 = direct_step(h);
     if (s0 != LBM_OK || --n == 0) return s0;
   }
+  while (use_resident(h, n)) {
+    const int m = n < kResidentMostSteps ? n : kResidentMostSteps;
+    LBM_CUDA(launch_resident(h->P, h->res, h->prm.store, (int)(h->step & 1), h->pop, h->ghost, h->flag,
+                             h->res_mem,
+                             reinterpret_cast<unsigned*>(static_cast<char*>(h->res_mem) + h->res_inbox),
+                             m, h->stream));
+    h->step += m;
+    n -= m;
+  }
+  if (n == 0) return LBM_OK;
   lbm_status s = ensure_graphs(h);
   if (s != LBM_OK) return s;
   if (h->step & 1) {
@@ -618,7 +677,7 @@ lbm_status lbm_synchronize(lbm_handle* h) {
   LBM_CUDA(cudaMemcpyAsync(&flag, h->flag, sizeof(flag), cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(cudaStreamSynchronize(h->stream));
   latch_flag(h, flag);
-  if (h->stalled) return fail(LBM_E_TIMEOUT, "a staged step gave up waiting for a bulk copy; re-init");
+  if (h->stalled) return fail(LBM_E_TIMEOUT, "a step gave up waiting for a bulk copy or a neighbouring block; re-init");
   if (h->nonfinite) return fail(LBM_E_NONFINITE, "non-finite moments detected");
   return LBM_OK;
 }
@@ -755,7 +814,7 @@ lbm_status finish_diag(lbm_handle* h, const double* r, unsigned flag, long long 
   out->eps_d_raw = 4.0 / 3.0 * r[14] / n;
   latch_flag(h, flag);
   if (r[6] > 0) h->nonfinite = true;
-  if (h->stalled) return fail(LBM_E_TIMEOUT, "a staged step gave up waiting for a bulk copy; re-init");
+  if (h->stalled) return fail(LBM_E_TIMEOUT, "a step gave up waiting for a bulk copy or a neighbouring block; re-init");
   if (h->nonfinite) return fail(LBM_E_NONFINITE, "non-finite moments detected");
   return LBM_OK;
 }
@@ -787,7 +846,7 @@ lbm_status lbm_step_diag(lbm_handle* h, int n, lbm_diag_t* out) {
   if (n < 1) return fail(LBM_E_INVAL, "n must be >= 1");
   if (!h->initialized) return fail(LBM_E_STATE, "lbm_step_diag before an init");
   if (h->nonfinite) return fail(LBM_E_NONFINITE, "non-finite moments were detected earlier");
-  if (h->stalled) return fail(LBM_E_TIMEOUT, "a staged step gave up waiting for a bulk copy; re-init");
+  if (h->stalled) return fail(LBM_E_TIMEOUT, "a step gave up waiting for a bulk copy or a neighbouring block; re-init");
   lbm_status st = ensure_diag_scratch(h);
   if (st != LBM_OK) return st;
   const int bx = effective_block(h);
@@ -990,7 +1049,7 @@ lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out) {
   LBM_CUDA(cudaMemcpyAsync(&flag, h->flag, sizeof(flag), cudaMemcpyDeviceToHost, h->stream));
   LBM_CUDA(cudaStreamSynchronize(h->stream));
   latch_flag(h, flag);
-  if (h->stalled) return fail(LBM_E_TIMEOUT, "a staged step gave up waiting for a bulk copy; re-init");
+  if (h->stalled) return fail(LBM_E_TIMEOUT, "a step gave up waiting for a bulk copy or a neighbouring block; re-init");
   if (out) {
     out->block_x = best_v >= kFirstStagedVariant ? 128 : effective_block(h);
     out->variant = best_v;
@@ -1036,11 +1095,13 @@ lbm_status lbm_set_kernel_config(lbm_handle* h, int block_x, int variant) {
     LBM_CUDA(staged_prepare(h->P, h->prm.store, variant, &grid));
     h->variant = variant;
     h->staged_grid = grid;
+    h->res_on = false;  // the caller asks for this form
     h->graphs_valid = false;
     return LBM_OK;
   }
   if (block_x < 32 || block_x > 128 || (block_x & 31))
     return fail(LBM_E_INVAL, "block_x must be 32, 64, 96 or 128");
+  h->res_on = false;
   h->block_x = block_x;
   h->variant = variant;
   h->graphs_valid = false;

@@ -74,6 +74,26 @@ inline long long step_diag_record_count(const DomainConst& P, int block_x) {
   return (long long)((P.nx + block_x - 1) / block_x) * P.ny * P.nz * (block_x / 32);
 }
 
+// Several steps of a small domain in one cooperative launch, the populations in registers
+// (step_resident.cu). A plan cuts the domain into bricks of b cells, g of them along each
+// axis, one block each.
+constexpr int kResidentMaxThreads = 384;  // cells of a brick at most: 170 registers a thread
+struct ResidentPlan {
+  int b[3], g[3];
+  int threads;  // of a block: the brick's cells rounded up to whole warps
+  int face;     // cells of the largest face through which bricks exchange
+  int blocks() const { return g[0] * g[1] * g[2]; }
+};
+// Chooses the bricks for `sms` blocks resident at once; false if the domain does not fit or
+// the plain kernel is faster.
+bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R);
+// Bytes of the bricks' inboxes (zeroed before the first launch; so are the epochs, one
+// word per block).
+size_t resident_inbox_bytes(const ResidentPlan& R, int store);
+cudaError_t launch_resident(const DomainConst& P, const ResidentPlan& R, int store, int parity,
+                            void* pop, const float* ghost, unsigned* flag, void* inbox,
+                            unsigned* epochs, int steps, cudaStream_t s);
+
 // Initial states (init.cu). kind: 0 TGV, 1 Riemann, 2 caller fields (rho, u, p),
 // 3 caller zeroth moments (14 fields). Host-computed FP32 constants; the device works
 // in FP32 only (the deviations from Q_ref are formed without cancellation).

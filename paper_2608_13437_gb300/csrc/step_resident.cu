@@ -1,0 +1,440 @@
+// Many steps of a small domain in one launch, with the populations held in registers.
+//
+// A grid of up to about 58 thousand cells (one brick of at most 384 cells per SM) is far
+// too small to be bound by memory: a step moves its 98 populations per cell through the
+// L2 for no reason but that launches end, and costs 3.1 us at 16 thousand cells, of which
+// about 1 us is the gap between two launches and most of the rest one chain of dependent
+// loads, arithmetic and stores. Here each block keeps a brick of cells for n steps, one
+// thread per cell with its 14 x 7 populations in registers (the plain step kernel's budget
+// of 170), and per step only what the lattice links carry moves: within the brick through
+// shared memory, between bricks through inboxes in global memory (the L2).
+//
+//   * Every directional population leaves as the words of the storage type (rounded as a
+//     plain step's store rounds it) and is decoded on arrival as a plain step's load does;
+//     collide_cell is the same code. So the state after n steps is the plain kernel's, bit
+//     for bit, for every storage type, rounding mode, streaming map and parity.
+//   * An inbox holds 16-byte packets of three words and a tag, the number of the step that
+//     sent them. Packets are written and read whole (128-bit scalar accesses), so a reader
+//     polls the packet itself until the tag is the current step's: one trip through the
+//     L2, no flags, no fences, no grid-wide barrier. A brick has two inboxes, for even and
+//     odd tags. A neighbour overwrites an inbox two steps later; by then it has received
+//     this brick's packets of the step between, which were sent after the inbox was read.
+//   * The same dependence orders memory at both ends of the launch: a brick stores its
+//     populations only after it has received a step's packets from its neighbours, which
+//     they send after they have loaded theirs, and a location is loaded and stored by one
+//     brick and its direct neighbours along that population's axis alone.
+//   * Launched cooperatively (every block resident, or the launch fails). A poll gives up
+//     after a bounded number of tries; the block then sets flag bit 2 and returns without
+//     storing, its neighbours run out the same way, and the host reports LBM_E_TIMEOUT.
+//   * Tags go on from each block's own step count in device memory, so a launch may be
+//     repeated (also by a graph) without the host's knowledge of it.
+#include <algorithm>
+
+#include "lbm_internal.h"
+
+namespace lbm {
+
+namespace {
+
+template <typename S>
+struct Words {
+  static constexpr int n = std::is_same<S, float>::value ? kF : kF / 2;  // of one direction
+  static constexpr int packets = (n + 2) / 3;
+};
+
+// The words of direction i's 14 fields, as store_dir stores them.
+template <typename S, bool SR>
+__device__ __forceinline__ void pack_dir(const DomainConst& P, const float (&d)[kF][kQ], int i,
+                                         Dither* dz, unsigned (&w)[Words<S>::n]) {
+  float v[kF];
+#pragma unroll
+  for (int k = 0; k < kF; ++k) v[k] = d[k][i];
+  if constexpr (std::is_same<S, float>::value) {
+#pragma unroll
+    for (int k = 0; k < kF; ++k) w[k] = __float_as_uint(v[k]);
+  } else {
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+      uint2 e;
+      if constexpr (SR) {
+        const unsigned r0 = dz->next(), r1 = dz->next();
+        e = Codec<S>::enc4_sr(v + 4 * g, P.inv_scale + 4 * g, r0, r1);
+      } else {
+        e = Codec<S>::enc4(v + 4 * g, P.inv_scale + 4 * g);
+      }
+      w[2 * g] = e.x;
+      w[2 * g + 1] = e.y;
+    }
+    if constexpr (SR) w[6] = Codec<S>::enc2_sr(v + 12, P.inv_scale + 12, dz->next());
+    else w[6] = Codec<S>::enc2(v + 12, P.inv_scale + 12);
+  }
+}
+
+// Decodes direction i's words, as load_cell decodes what it loads.
+template <typename S>
+__device__ __forceinline__ void unpack_dir(const DomainConst& P, const unsigned (&w)[Words<S>::n],
+                                           float (&d)[kF][kQ], int i) {
+  float v[kF];
+  if constexpr (std::is_same<S, float>::value) {
+#pragma unroll
+    for (int k = 0; k < kF; ++k) v[k] = __uint_as_float(w[k]);
+  } else {
+#pragma unroll
+    for (int g = 0; g < 3; ++g)
+      Codec<S>::dec4(make_uint2(w[2 * g], w[2 * g + 1]), P.scale + 4 * g, v + 4 * g);
+    Codec<S>::dec2(w[6], P.scale + 12, v + 12);
+  }
+#pragma unroll
+  for (int k = 0; k < kF; ++k) d[k][i] = v[k];
+}
+
+// A direction's words as the groups of 4 + 4 + 4 + 2 fields of the population layout
+// and of the exchange through shared memory.
+template <typename S>
+__device__ __forceinline__ typename Codec<S>::V4 words4(const unsigned* w, int g) {
+  if constexpr (std::is_same<S, float>::value)
+    return make_float4(__uint_as_float(w[4 * g]), __uint_as_float(w[4 * g + 1]),
+                       __uint_as_float(w[4 * g + 2]), __uint_as_float(w[4 * g + 3]));
+  else
+    return make_uint2(w[2 * g], w[2 * g + 1]);
+}
+template <typename S>
+__device__ __forceinline__ typename Codec<S>::V2 words2(const unsigned* w) {
+  if constexpr (std::is_same<S, float>::value)
+    return make_float2(__uint_as_float(w[12]), __uint_as_float(w[13]));
+  else
+    return w[6];
+}
+template <typename S>
+__device__ __forceinline__ void from_groups(const typename Codec<S>::V4 (&a)[3],
+                                            typename Codec<S>::V2 b,
+                                            unsigned (&w)[Words<S>::n]) {
+  if constexpr (std::is_same<S, float>::value) {
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+      w[4 * g] = __float_as_uint(a[g].x);
+      w[4 * g + 1] = __float_as_uint(a[g].y);
+      w[4 * g + 2] = __float_as_uint(a[g].z);
+      w[4 * g + 3] = __float_as_uint(a[g].w);
+    }
+    w[12] = __float_as_uint(b.x);
+    w[13] = __float_as_uint(b.y);
+  } else {
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+      w[2 * g] = a[g].x;
+      w[2 * g + 1] = a[g].y;
+    }
+    w[6] = b;
+  }
+}
+
+// Inbox packets: 128-bit scalar accesses, so the three words and the tag arrive together.
+__device__ __forceinline__ void packet_store(uint4* p, unsigned a, unsigned b, unsigned c, unsigned tag) {
+  const unsigned long long lo = a | ((unsigned long long)b << 32), hi = c | ((unsigned long long)tag << 32);
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\t"
+      "st.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p), "l"(lo), "l"(hi)
+      : "memory");
+}
+__device__ __forceinline__ uint4 packet_load(const uint4* p) {
+  unsigned long long lo, hi;
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\t"
+      "mov.b128 {%0, %1}, t;\n\t}"
+      : "=l"(lo), "=l"(hi)
+      : "l"(p)
+      : "memory");
+  return make_uint4((unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32));
+}
+
+// Tries of one poll before a block gives up: each is a trip through the L2 (about half a
+// microsecond), so about a second.
+constexpr int kMaxPolls = 1 << 21;
+
+template <typename S, bool SR>
+__global__ void __launch_bounds__(kResidentMaxThreads, 1)
+    k_resident(const DomainConst P, const ResidentPlan R, S* __restrict__ pop,
+               const float* __restrict__ ghost, unsigned* __restrict__ flag,
+               uint4* __restrict__ inbox, unsigned* __restrict__ epochs, int parity0, int steps) {
+  using V4 = typename Codec<S>::V4;
+  using V2 = typename Codec<S>::V2;
+  constexpr int NW = Words<S>::n, NP = Words<S>::packets;
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int T = blockDim.x, tid = threadIdx.x;
+  V4* const s4 = reinterpret_cast<V4*>(smem);              // [6][3][T]
+  V2* const s2 = reinterpret_cast<V2*>(s4 + 6 * 3 * T);    // [6][T]
+  uint2* const table = reinterpret_cast<uint2*>(s2 + 6 * T);  // [packet sets of the brick]
+  // brick and cell
+  const int bx = blockIdx.x % R.g[0], by = blockIdx.x / R.g[0] % R.g[1],
+            bz = blockIdx.x / (R.g[0] * R.g[1]);
+  const int lx = tid % R.b[0], ly = tid / R.b[0] % R.b[1], lz = tid / (R.b[0] * R.b[1]);
+  const int x = bx * R.b[0] + lx, y = by * R.b[1] + ly, z = bz * R.b[2] + lz;
+  const bool active = lz < R.b[2] && x < P.nx && y < P.ny && z < P.nz;
+  // Per direction i = 1..6: where the population leaving along i goes: the thread of this
+  // brick that owns the next cell, or kOut for the neighbouring brick.
+  constexpr int kOut = 0xFFFF;
+  int to[6];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int l = a == 0 ? lx : (a == 1 ? ly : lz);
+    const int stride = a == 0 ? 1 : (a == 1 ? R.b[0] : R.b[0] * R.b[1]);
+    const int first = (a == 0 ? bx : (a == 1 ? by : bz)) * R.b[a];
+    const int n = a == 0 ? P.nx : (a == 1 ? P.ny : P.nz);
+    const int width = min(R.b[a], n - first);  // of this brick
+    const bool whole = R.g[a] == 1;            // the brick spans the axis: wrap inside
+    to[2 * a] = l + 1 < width ? tid + stride : (whole ? tid - (width - 1) * stride : kOut);
+    to[2 * a + 1] = l > 0 ? tid - stride : (whole ? tid + (width - 1) * stride : kOut);
+  }
+  // offset of packet 0 of direction i to the face cell f of brick b's inbox 0
+  auto slot = [&](int b, int i, int f) { return (unsigned)((b * 12 + (i - 1)) * NP * R.face + f); };
+  auto neighbour = [&](int i) {  // the brick that direction i leads to
+    const int a = (i - 1) >> 1, s = (i & 1) ? 1 : -1;
+    const int c = a == 0 ? bx : (a == 1 ? by : bz);
+    int m = c + s;
+    if (m == R.g[a]) m = 0;
+    if (m < 0) m = R.g[a] - 1;
+    const int step = a == 0 ? 1 : (a == 1 ? R.g[0] : R.g[0] * R.g[1]);
+    return (int)blockIdx.x + (m - c) * step;
+  };
+
+  // Table of the packet sets that arrive from outside: inbox offset, and direction (less
+  // one) and thread of the receiving cell.
+  int n_in = 0;
+  {
+    const int w[3] = {min(R.b[0], P.nx - bx * R.b[0]), min(R.b[1], P.ny - by * R.b[1]),
+                      min(R.b[2], P.nz - bz * R.b[2])};
+    const int s[3] = {1, R.b[0], R.b[0] * R.b[1]};  // thread strides
+    for (int a = 0; a < 3; ++a) {
+      if (R.g[a] == 1) continue;
+      const int u = a == 0 ? 1 : 0, v = a == 2 ? 1 : 2;  // the face's axes
+      for (int e = tid; e < w[u] * w[v]; e += T) {
+        const int lu = e % w[u], lv = e / w[u], f = lu + R.b[u] * lv;
+        const int at = lu * s[u] + lv * s[v];
+        // along +a into the cells at the low end, along -a at the high end
+        table[n_in + 2 * e] = make_uint2(slot(blockIdx.x, 2 * a + 1, f), (2u * a) << 16 | at);
+        table[n_in + 2 * e + 1] =
+            make_uint2(slot(blockIdx.x, 2 * a + 2, f), (2u * a + 1) << 16 | (at + (w[a] - 1) * s[a]));
+      }
+      n_in += 2 * w[u] * w[v];
+    }
+  }
+  __syncthreads();
+
+  float d[kF][kQ];
+  const CellIndex c = make_index(P, x, y, z);
+  const unsigned epoch = epochs[blockIdx.x];
+  if (active) {
+    if (parity0) load_cell<1, false, S>(P, pop, nullptr, c, d);
+    else load_cell<0, false, S>(P, pop, nullptr, c, d);
+  }
+  bool bad = false;
+  // Where the state is stored after the last step: the read position of the new parity.
+  const int parity1 = (parity0 + steps) & 1;
+  auto store_words = [&](int i, const unsigned (&w)[NW]) {
+    const long long cell = src_cell(P, c, parity1, i);
+    if (!LBM_CHECK(P, cell >= 0 && cell < P.ntile * kTile)) return;
+    S* base = pop + tile_start(cell);
+    const int lane = (int)(cell & (kTile - 1));
+    const int sl = parity1 ? opp(i) : i;
+#pragma unroll
+    for (int g = 0; g < 3; ++g) *reinterpret_cast<V4*>(base + group_offset(sl, g, lane)) = words4<S>(w, g);
+    *reinterpret_cast<V2*>(base + group_offset(sl, 3, lane)) = words2<S>(w);
+  };
+
+#pragma unroll 1
+  for (int t = 0; t < steps; ++t) {
+    const unsigned tag = epoch + (unsigned)t + 1u;
+    const bool last = t + 1 == steps;
+    if (active) {
+      if (P.bc_x) {  // held x ends: the inward populations come from the ghost layer
+        if (x == 0) {
+#pragma unroll
+          for (int k = 0; k < kF; ++k) d[k][1] = ghost_value(P, ghost, c, k, 1);
+        }
+        if (x == P.nx - 1) {
+#pragma unroll
+          for (int k = 0; k < kF; ++k) d[k][2] = ghost_value(P, ghost, c, k, 2);
+        }
+      }
+      const float probe = collide_cell<false>(P, d, nullptr);
+      bad = bad || !isfinite(probe);
+      [[maybe_unused]] Dither dz(0, 0.0f, 0.0f);
+      if constexpr (SR) dz = Dither(c.own, d[0][0], d[4][0]);
+#pragma unroll
+      for (int i = 0; i < kQ; ++i) {
+        unsigned w[NW];
+        pack_dir<S, SR>(P, d, i, &dz, w);
+        if (i == 0) {
+          if (last) store_words(0, w);
+          else if constexpr (!std::is_same<S, float>::value) unpack_dir<S>(P, w, d, 0);
+          continue;
+        }
+        const int dst = to[i - 1];
+        if (dst == kOut) {
+          // the destination cell has the same place on its brick's face
+          const int f = i < 3 ? ly + R.b[1] * lz : (i < 5 ? lx + R.b[0] * lz : lx + R.b[0] * ly);
+          uint4* p = inbox + slot(neighbour(i), i, f) + (tag & 1u) * (6u * NP * R.face);
+#pragma unroll
+          for (int q = 0; q < NP; ++q)
+            packet_store(p + (size_t)q * R.face, w[3 * q], 3 * q + 1 < NW ? w[3 * q + 1] : tag,
+                         3 * q + 2 < NW ? w[3 * q + 2] : tag, tag);
+        } else {
+#pragma unroll
+          for (int g = 0; g < 3; ++g) s4[((i - 1) * 3 + g) * T + dst] = words4<S>(w, g);
+          s2[(i - 1) * T + dst] = words2<S>(w);
+        }
+      }
+    }
+    // What the neighbours send: thread tid fetches packet sets tid, tid + T, ... of the brick
+    // (all packets of one cell and direction), so the polls of all faces are one trip
+    // through the L2 instead of one per direction, and puts them where the exchange within
+    // the brick would.
+    bool dead = false;
+    for (int e = tid; e < n_in; e += T) {
+      const uint2 in = table[e];
+      const uint4* p = inbox + in.x + (tag & 1u) * (6u * NP * R.face);
+      unsigned w[3 * NP];
+      for (int tries = 0;; ++tries) {
+        uint4 m[NP];
+#pragma unroll
+        for (int q = 0; q < NP; ++q) m[q] = packet_load(p + (size_t)q * R.face);
+        bool ok = true;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+          // every word of a packet is used, so that its load stays one access: with the
+          // spare words of the last packet ignored the load was narrowed and the packet
+          // could be read half old, half new
+          ok = ok && m[q].w == tag;
+          if (3 * q + 1 >= NW) ok = ok && m[q].y == tag;
+          if (3 * q + 2 >= NW) ok = ok && m[q].z == tag;
+        }
+        if (ok || dead || tries >= kMaxPolls) {
+          dead = dead || !ok;
+#pragma unroll
+          for (int q = 0; q < NP; ++q) {
+            w[3 * q] = m[q].x;
+            w[3 * q + 1] = m[q].y;
+            w[3 * q + 2] = m[q].z;
+          }
+          break;
+        }
+      }
+#pragma unroll
+      for (int g = 0; g < 3; ++g) s4[(in.y >> 16) * 3 * T + g * T + (in.y & 0xFFFFu)] = words4<S>(w, g);
+      s2[(in.y >> 16) * T + (in.y & 0xFFFFu)] = words2<S>(w);
+    }
+    __syncthreads();
+    if (active) {
+#pragma unroll
+      for (int i = 1; i < kQ; ++i) {
+        V4 a[3];
+#pragma unroll
+        for (int g = 0; g < 3; ++g) a[g] = s4[((i - 1) * 3 + g) * T + tid];
+        unsigned w[NW];
+        from_groups<S>(a, s2[(i - 1) * T + tid], w);
+        if (last) store_words(i, w);
+        else unpack_dir<S>(P, w, d, i);
+      }
+    }
+    // everyone is done with the exchange buffer; a block whose wait ran out stops here
+    if (__syncthreads_or(dead)) {
+      if (tid == 0) atomicOr(flag, 2u);
+      return;
+    }
+  }
+  if (bad) atomicOr(flag, 1u);
+  if (tid == 0) epochs[blockIdx.x] = epoch + (unsigned)steps;
+}
+
+// Shared memory of a block: six directions of every cell, and the table (at most six
+// packet sets a cell).
+template <typename S>
+constexpr size_t smem_bytes(int threads) {
+  return (size_t)threads * 6 * (kF * sizeof(S) + sizeof(uint2));
+}
+
+template <typename S, bool SR>
+cudaError_t launch_t(const DomainConst& P, const ResidentPlan& R, void* pop, const float* ghost,
+                     unsigned* flag, void* inbox, unsigned* epochs, int parity, int steps,
+                     cudaStream_t s) {
+  const size_t smem = smem_bytes<S>(R.threads);
+  cudaError_t e = cudaFuncSetAttribute(k_resident<S, SR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem_bytes<S>(kResidentMaxThreads));
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(R.blocks());
+  cfg.blockDim = dim3(R.threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeCooperative;
+  attr.val.cooperative = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_resident<S, SR>, P, R, static_cast<S*>(pop), ghost, flag,
+                            static_cast<uint4*>(inbox), epochs, parity, steps);
+}
+
+}  // namespace
+
+bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R) {
+  if (!P.collide || P.ncell > (long long)sms * kResidentMaxThreads) return false;
+  const int n[3] = {P.nx, P.ny, P.nz};
+  long long best = -1;
+  for (int bx = 1; bx <= std::min(n[0], kResidentMaxThreads); ++bx) {
+    const int gx = (n[0] + bx - 1) / bx;
+    if (gx > sms) continue;
+    for (int by = 1; by <= std::min(n[1], kResidentMaxThreads / bx); ++by) {
+      const int gy = (n[1] + by - 1) / by;
+      if (gx * gy > sms) continue;
+      for (int bz = 1; bz <= std::min(n[2], kResidentMaxThreads / (bx * by)); ++bz) {
+        const int gz = (n[2] + bz - 1) / bz;
+        if (gx * gy * gz > sms) continue;
+        const int face[3] = {gx > 1 ? by * bz : 0, gy > 1 ? bx * bz : 0, gz > 1 ? bx * by : 0};
+        // Nanoseconds of a step, fitted to a sweep of 80 bricks of nine domains (FP32, within
+        // about 10 %): one warp's latency, the issue of the brick's warps, a trip to the
+        // neighbours along each axis that leaves the brick, and one more poll for every
+        // further packet set a thread fetches.
+        const long long warps = (bx * by * bz + 31) / 32;
+        const long long sets = 2LL * (face[0] + face[1] + face[2]), threads = 32 * warps;
+        long long cost = 1200 + 150 * warps;
+        for (int a = 0; a < 3; ++a) cost += face[a] ? 300 : 0;
+        if (sets > 0) cost += 400 * ((sets + threads - 1) / threads - 1);
+        if (best < 0 || cost < best) {
+          best = cost;
+          *R = ResidentPlan{{bx, by, bz}, {gx, gy, gz}, (int)(32 * warps),
+                            std::max(1, std::max(face[0], std::max(face[1], face[2])))};
+        }
+      }
+    }
+  }
+  // Against the plain kernel's nanoseconds at these sizes, fitted to the same domains: 2.2 us
+  // at 4 thousand cells, 3.8 at 33 thousand (FP32); 16-bit storage 2.4-2.6 and 3.0-3.1 us,
+  // and its resident form is 0.1 to 0.4 us below the model. Resident, FP32: 2.06 us at
+  // 1024 x 4 x 4 (plain 3.08), 3.21 at 32^3 (3.78), 4.47 at 38^3 (6.17), 2.48 at 16^3 (2.18).
+  if (best < 0) return false;
+  return store == 0 ? best + 150 < 2050 + 52 * P.ncell / 1000 : best - 200 < 2300 + 25 * P.ncell / 1000;
+}
+
+size_t resident_inbox_bytes(const ResidentPlan& R, int store) {
+  const int packets = store == 0 ? Words<float>::packets : Words<__half>::packets;
+  return (size_t)R.blocks() * 2 * 6 * packets * R.face * sizeof(uint4);
+}
+
+cudaError_t launch_resident(const DomainConst& P, const ResidentPlan& R, int store, int parity,
+                            void* pop, const float* ghost, unsigned* flag, void* inbox,
+                            unsigned* epochs, int steps, cudaStream_t s) {
+  cudaError_t e;
+  if (store == 0) e = launch_t<float, false>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
+  else if (store == 1)
+    e = P.sround ? launch_t<__half, true>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s)
+                 : launch_t<__half, false>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
+  else
+    e = P.sround ? launch_t<__nv_bfloat16, true>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s)
+                 : launch_t<__nv_bfloat16, false>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
+}  // namespace lbm

@@ -1,0 +1,104 @@
+"""Small domains: lbm_step takes many steps in one launch with the populations held on the
+chip. The result has to be the one-launch-per-step kernel's (use_graphs = 0), bit for bit."""
+import numpy as np
+import pytest
+
+from paper_2608_13437_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_13437_gb300 import build, lbm as L
+    build.build()
+    L.lib()
+    return L
+
+
+# shapes: the configurations in use, bricks that do not divide a side, one brick, two bricks
+# along an axis (both neighbours are the same one), sides of one and two cells, long rows,
+# the largest domain that fits 152 SMs and one just above it (the plain kernel's, as are
+# the sizes at which the plain kernel is the faster one).
+SHAPES = [(32, 32, 32), (20, 12, 9), (37, 6, 5), (1, 1, 1), (2, 1, 1), (1, 1, 700), (385, 1, 1),
+          (5, 4, 3), (64, 8, 4), (33, 31, 35), (7, 61, 3), (1000, 3, 2), (48, 32, 38), (38, 38, 40)]
+FORMS = [("f32", 0, 0), ("f32", 0, 1), ("f16", 0, 0), ("f16", 1, 1), ("bf16", 1, 0), ("bf16", 0, 1)]
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("held", [0, 1])
+def test_resident_steps_equal_plain_steps(lbm, shape, held):
+    nx, ny, nz = shape
+    for j, (store, sr, streaming) in enumerate(FORMS):
+        p = inputs.sod_params(64) if held else inputs.tgv_params(16)
+        p.update(nx=nx, ny=ny, nz=nz, dx=2 * np.pi / 40, streaming=streaming, stochastic_round=sr)
+        if not held:
+            p.update(sutherland=j & 1, f_mu=0.3, J_min=1e-3, tau_R=0.05, tau_q=0.05)
+        s = inputs.random_smooth_state(nx, ny, nz, seed=11 + j, amp=0.15)
+        a, b = lbm.Domain(p, store=store), lbm.Domain(p, store=store, use_graphs=False)
+        for d in (a, b):
+            d.init_fields(s["rho"], s["ux"], s["uy"] + 0.1, s["uz"], s["p"])
+        for n in (8, 9, 1, 8, 11, 3):  # both parities at either end of a launch, plain steps between
+            a.step(n)
+            b.step(n)
+        a.synchronize()
+        assert a.step_count == b.step_count == 40
+        assert np.array_equal(a.populations("native"), b.populations("native")), (store, sr, streaming)
+        whole = nx * ny * nz % 32 == 0  # otherwise the last tile has lanes that nothing writes
+        if whole:
+            assert lbm_equal(a.buffer, b.buffer), (store, sr, streaming)
+        a.close()
+        b.close()
+
+
+def lbm_equal(a, b):
+    return bool((a == b).all())
+
+
+def test_resident_flags_nonfinite_and_recovers(lbm):
+    """A NaN put into one cell is reported at the next synchronising call, steps are refused,
+    and a re-init gives a fresh handle's result."""
+    p = inputs.tgv_params(32)
+    d, e = lbm.Domain(p), lbm.Domain(p, use_graphs=False)
+    d.init_tgv(1.0, 1.25, 1.0)
+    f = d.populations(np.float64)
+    f[0, 0, 3, 4, 5] = np.nan
+    d.set_populations(f)
+    d.step(10)
+    with pytest.raises(lbm.LbmError) as ei:
+        d.synchronize()
+    assert ei.value.status == lbm.LBM_E_NONFINITE
+    with pytest.raises(lbm.LbmError):
+        d.step(8)
+    for h in (d, e):
+        h.init_tgv(1.0, 1.25, 1.0)
+        h.step(9)
+    assert np.array_equal(d.populations("native"), e.populations("native"))
+    d.close()
+    e.close()
+
+
+def test_resident_handles_on_two_streams(lbm):
+    """Two small domains stepped from two streams at once: each equals its own plain run."""
+    import torch
+    p = inputs.tgv_params(32)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    doms, refs = [], []
+    for j, st in enumerate(streams):
+        with torch.cuda.stream(st):
+            doms.append(lbm.Domain(p))
+            doms[-1].init_tgv(1.0, 1.0 + 0.1 * j, 1.0)
+    for _ in range(5):
+        for d in doms:
+            d.step(40)
+    for j, d in enumerate(doms):
+        d.synchronize()
+        r = lbm.Domain(p, use_graphs=False)
+        r.init_tgv(1.0, 1.0 + 0.1 * j, 1.0)
+        r.step(200)
+        assert np.array_equal(d.populations("native"), r.populations("native"))
+        r.close()
+        d.close()
