@@ -4,12 +4,39 @@ physical space, and the shell-averaged kinetic-energy spectrum normalised so tha
 sum_k E(k) = <|u|^2> / 2. Inputs are the primitive fields that lbm_moments(LBM_MOM_PRIM)
 writes (rho, u_x, u_y, u_z, T, p), as a device tensor (6, nz, ny, nx), on a periodic box
 of side L_box per axis.
+
+FP64 tensors on the GPU take half spectra (real transforms) and the passes of
+lbm_spectral.h: three transforms forward, curl and divergence formed in spectral space
+(four fields instead of the nine gradients), four back, one pass for the means. The FP64
+rate bounds the transforms on this part, so their number is what counts. Other tensors
+(CPU, FP32, under autograd or a functional transform) take plain tensor operations.
 """
 from __future__ import annotations
 
 import math
 
 T_SUTHERLAND = 0.4042
+_DOUBLES = 2 + 2 * 1216  # LBM_SPECTRAL_DOUBLES
+_MOST_SHELLS = 6000
+
+
+def _on_device(t):
+    """Whether the tensor's values alone are wanted and the library's passes can read it: a
+    plain FP64 CUDA tensor, nothing recording, transforming or capturing operations."""
+    import torch
+    from torch.autograd import forward_ad
+    if (type(t) is not torch.Tensor or not t.is_cuda or t.dtype != torch.float64
+            or (t.requires_grad and torch.is_grad_enabled()) or not 0 < t.numel() < 1 << 31):
+        return False
+    peek = getattr(torch._C._functorch, "peek_interpreter_stack", None)
+    return not (torch.compiler.is_compiling() or peek is None or peek() is not None
+                or getattr(forward_ad, "_current_level", -1) >= 0
+                or torch._C._len_torch_dispatch_stack()
+                or torch.cuda.is_current_stream_capturing())
+
+
+def _numbers(*values):
+    return all(isinstance(v, (int, float)) for v in values)
 
 
 def _k(n, L_box, device, dtype):
@@ -38,6 +65,9 @@ def gradients(u, L_box=2 * math.pi):
 def dissipation(prim, mu, T_ref, sutherland, rho_ref, L_box=2 * math.pi):
     """(eps_s, eps_d) of Eq. 7 from primitive fields (6, nz, ny, nx) (FP64 recommended)."""
     import torch
+    if (prim.ndim == 4 and len(prim) >= 5 and _numbers(mu, T_ref, rho_ref, L_box)
+            and _on_device(prim)):
+        return _dissipation_device(prim, mu, T_ref, sutherland, rho_ref, L_box)
     g = gradients(prim[1:4], L_box)
     wx, wy, wz = g[1, 2] - g[2, 1], g[2, 0] - g[0, 2], g[0, 1] - g[1, 0]
     div = g[0, 0] + g[1, 1] + g[2, 2]
@@ -52,10 +82,41 @@ def dissipation(prim, mu, T_ref, sutherland, rho_ref, L_box=2 * math.pi):
     return float(eps_s), float(eps_d)
 
 
+def _dissipation_device(prim, mu, T_ref, sutherland, rho_ref, L_box):
+    import torch
+
+    from . import lbm
+    nz, ny, nx = prim.shape[1:]
+    with torch.cuda.device(prim.device):
+        L, stream = lbm.lib(), torch.cuda.current_stream().cuda_stream
+        uh = torch.fft.rfftn(prim[1:4], dim=(1, 2, 3)).contiguous()
+        wh = uh.new_empty((4,) + tuple(uh.shape[1:]))
+        lbm.check(L.lbm_spectral_curl_div(uh.data_ptr(), wh.data_ptr(), nx, ny, nz,
+                                          2 * math.pi / L_box, stream))
+        w = torch.fft.irfftn(wh, s=(nz, ny, nx), dim=(1, 2, 3), norm="forward").contiguous()
+        T = prim[4].contiguous()
+        out = torch.empty(_DOUBLES, dtype=torch.float64, device=prim.device)
+        lbm.check(L.lbm_spectral_dissipation(w.data_ptr(), T.data_ptr(), nx * ny * nz, mu, T_ref,
+                                             int(bool(sutherland)), out.data_ptr(), stream))
+        s, d = out[:2].tolist()
+    return s / rho_ref, 4.0 / 3.0 * d / rho_ref
+
+
 def energy_spectrum(u, L_box=2 * math.pi):
     """(k, E(k)) over unit-width shells of |k| L; sum(E) = <|u|^2> / 2."""
     import torch
     nz, ny, nx = u.shape[1:]
+    if u.ndim == 4 and len(u) == 3 and _numbers(L_box) and _on_device(u):
+        from . import lbm
+        L = lbm.lib()
+        shells = L.lbm_spectral_shell_count(nx, ny, nz)
+        if shells <= _MOST_SHELLS:
+            with torch.cuda.device(u.device):
+                uh = torch.fft.rfftn(u, dim=(1, 2, 3)).contiguous()
+                e = torch.zeros(shells, dtype=u.dtype, device=u.device)
+                lbm.check(L.lbm_spectral_shells(uh.data_ptr(), nx, ny, nz, e.data_ptr(), shells,
+                                                torch.cuda.current_stream().cuda_stream))
+                return torch.arange(shells, device=u.device), e
     dt = u.dtype
     kx = _k_full(nx, L_box, u.device, dt).view(1, 1, nx)
     ky = _k_full(ny, L_box, u.device, dt).view(1, ny, 1)

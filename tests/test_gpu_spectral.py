@@ -1,0 +1,58 @@
+"""The device passes of the spectral diagnostics against the FP64 oracle and against the
+tensor operations that other tensors take (the same function on the CPU)."""
+import math
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2608_13437_gb300 import build, lbm as L
+    build.build()
+    L.lib()
+    return L
+
+
+# odd, even and unit sides; more modes than one wave of blocks; rows of one mode
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 2, 2), (3, 5, 7), (4, 6, 9), (9, 4, 2), (16, 16, 16),
+                                   (33, 20, 31), (5, 1, 64), (72, 70, 66)])
+@pytest.mark.parametrize("sutherland", [0, 1])
+def test_device_passes_match_oracle_and_tensor_path(lbm, shape, sutherland):
+    """Tolerance: 1e-12 of the largest value (FP64 transforms and sums, a few hundred ulp)."""
+    import torch
+    from oracle import spectral as ospec
+    from paper_2608_13437_gb300 import spectral
+    rng = np.random.default_rng(sum(shape))
+    prim = np.abs(rng.standard_normal((6,) + shape)) + 0.2
+    prim[1:4] = rng.standard_normal((3,) + shape)
+    L_box, mu, T_ref, rho = 2 * math.pi * 1.3, 2e-3, 0.7, 1.1
+    dev = torch.from_numpy(prim).cuda()
+    es, ed = spectral.dissipation(dev, mu, T_ref, sutherland, rho, L_box)
+    for ref in (spectral.dissipation(torch.from_numpy(prim), mu, T_ref, sutherland, rho, L_box),
+                ospec.dissipation(prim[1:4], prim[4], mu, T_ref, sutherland, rho, L_box)):
+        scale = max(abs(ref[0]), abs(ref[1]), 1e-300)
+        assert abs(es - ref[0]) <= 1e-12 * scale and abs(ed - ref[1]) <= 1e-12 * scale
+    k, e = spectral.energy_spectrum(dev[1:4], L_box)
+    kc, ec = spectral.energy_spectrum(torch.from_numpy(prim)[1:4], L_box)
+    assert torch.equal(k.cpu(), kc) and e.dtype == ec.dtype and e.device == dev.device
+    assert float((e.cpu() - ec).abs().max()) <= 1e-12 * float(ec.max())
+    # a strided view takes the same passes
+    strided = torch.empty((12,) + shape, dtype=torch.float64, device="cuda")[::2]
+    strided.copy_(dev)
+    assert spectral.dissipation(strided, mu, T_ref, sutherland, rho, L_box) == pytest.approx((es, ed), rel=1e-12)
+
+
+def test_tensors_under_autograd_take_tensor_operations(lbm):
+    """E(k) of a velocity that requires a gradient stays differentiable."""
+    import torch
+    from paper_2608_13437_gb300 import spectral
+    u = torch.randn(3, 6, 6, 6, dtype=torch.float64, device="cuda", requires_grad=True)
+    _, e = spectral.energy_spectrum(u)
+    e.sum().backward()
+    assert torch.allclose(u.grad, u.detach() / 216, rtol=1e-9, atol=1e-12)
