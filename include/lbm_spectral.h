@@ -18,25 +18,28 @@
 extern "C" {
 #endif
 
-/* Half spectra wh[4] of (curl u)_x, (curl u)_y, (curl u)_z and div u, divided by the
- * number of points, from the half spectra uh[3] of u. k0 = 2 pi / box side; the Nyquist
- * wavenumber of an even axis counts as 0 (no derivative of that mode of a real field). */
-lbm_status lbm_spectral_curl_div(const void* uh, void* wh, int nx, int ny, int nz, double k0,
-                                 void* cuda_stream);
+/* Spectra wh[2] of (curl u)_x + i (curl u)_y and (curl u)_z + i div u over the whole
+ * (nz, ny, nx) grid, divided by the number of points, from the unnormalised spectrum zh of
+ * u_x + i u_y over the whole grid and the half spectrum ch of u_z (a complex transform
+ * carries two real fields). k0 = 2 pi / box side; the Nyquist wavenumber of an even axis
+ * counts as 0 (no derivative of that mode of a real field). */
+lbm_status lbm_spectral_curl_div(const void* zh, const void* ch, void* wh, int nx, int ny, int nz,
+                                 double k0, void* cuda_stream);
 
-/* out[0] = mean of m |w|^2, out[1] = mean of m d^2 over n points, from w[4][n] =
- * (curl, div) in physical space and the temperature T[n]; m = mu, or Sutherland's law with
- * t = T/T_ref if sutherland. out must hold LBM_SPECTRAL_DOUBLES doubles (scratch). */
+/* out[0] = mean of m |w|^2, out[1] = mean of m d^2 over n points, from the complex fields
+ * w[2][n] = (w_x + i w_y, w_z + i d) in physical space and the temperature T[n]; m = mu,
+ * or Sutherland's law with t = T/T_ref if sutherland. out must hold LBM_SPECTRAL_DOUBLES
+ * doubles (scratch). */
 #define LBM_SPECTRAL_DOUBLES (2 + 2 * 1216)
-lbm_status lbm_spectral_dissipation(const double* w, const double* T, long long n, double mu,
+lbm_status lbm_spectral_dissipation(const void* w, const double* T, long long n, double mu,
                                     double T_ref, int sutherland, double* out, void* cuda_stream);
 
-/* Adds |uh_b / N|^2 / 2 of all N modes of the three components to the unit-width shells
+/* Adds |u_b / N|^2 / 2 of all N modes of the three components (zh, ch as above) to the shells
  * e[round(|m|)] (m: integer wavenumber vector); e must be zeroed, and nshell = 1 + the
  * largest shell of the grid (lbm_spectral_shell_count, at most 6000). */
 int lbm_spectral_shell_count(int nx, int ny, int nz);
-lbm_status lbm_spectral_shells(const void* uh, int nx, int ny, int nz, double* e, int nshell,
-                               void* cuda_stream);
+lbm_status lbm_spectral_shells(const void* zh, const void* ch, int nx, int ny, int nz, double* e,
+                               int nshell, void* cuda_stream);
 
 #ifdef __cplusplus
 }

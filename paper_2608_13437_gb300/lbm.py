@@ -117,11 +117,11 @@ _SIGNATURES = {
     "lbm_batch_autotune": (_IP, [_VP, _IP, ctypes.POINTER(_IP), ctypes.POINTER(_IP),
                                  ctypes.POINTER(ctypes.c_float), ctypes.POINTER(_IP)]),
     "lbm_batch_set_prefetch": (_IP, [_VP, _IP]),
-    "lbm_spectral_curl_div": (_IP, [_VP, _VP, _IP, _IP, _IP, ctypes.c_double, _VP]),
+    "lbm_spectral_curl_div": (_IP, [_VP, _VP, _VP, _IP, _IP, _IP, ctypes.c_double, _VP]),
     "lbm_spectral_dissipation": (_IP, [_VP, _VP, ctypes.c_longlong, ctypes.c_double, ctypes.c_double,
                                        _IP, _VP, _VP]),
     "lbm_spectral_shell_count": (_IP, [_IP, _IP, _IP]),
-    "lbm_spectral_shells": (_IP, [_VP, _IP, _IP, _IP, _VP, _IP, _VP]),
+    "lbm_spectral_shells": (_IP, [_VP, _VP, _IP, _IP, _IP, _VP, _IP, _VP]),
     "lbm_check_count": (_IP, [_VP, ctypes.POINTER(ctypes.c_ulonglong)]),
     "lbm_batch_check_count": (_IP, [_VP, ctypes.POINTER(ctypes.c_ulonglong)]),
 }

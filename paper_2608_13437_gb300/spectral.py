@@ -5,10 +5,11 @@ sum_k E(k) = <|u|^2> / 2. Inputs are the primitive fields that lbm_moments(LBM_M
 writes (rho, u_x, u_y, u_z, T, p), as a device tensor (6, nz, ny, nx), on a periodic box
 of side L_box per axis.
 
-FP64 tensors on the GPU take half spectra (real transforms) and the passes of
-lbm_spectral.h: three transforms forward, curl and divergence formed in spectral space
-(four fields instead of the nine gradients), four back, one pass for the means. The FP64
-rate bounds the transforms on this part, so their number is what counts. Other tensors
+FP64 tensors on the GPU take the passes of lbm_spectral.h: curl and divergence are formed
+in spectral space (four fields instead of nine gradients), and a complex transform carries
+two real fields, so a sample takes one complex and one real transform forward and two
+complex ones back, and one pass for the means. The FP64 rate bounds the transforms on
+this part (364 us for a complex one at 128^3), so their number counts. Other tensors
 (CPU, FP32, under autograd or a functional transform) take plain tensor operations.
 """
 from __future__ import annotations
@@ -82,6 +83,13 @@ def dissipation(prim, mu, T_ref, sutherland, rho_ref, L_box=2 * math.pi):
     return float(eps_s), float(eps_d)
 
 
+def _packed_spectra(u):
+    """Spectrum of u_x + i u_y over the whole grid and half spectrum of u_z."""
+    import torch
+    return (torch.fft.fftn(torch.complex(u[0], u[1])).contiguous(),
+            torch.fft.rfftn(u[2]).contiguous())
+
+
 def _dissipation_device(prim, mu, T_ref, sutherland, rho_ref, L_box):
     import torch
 
@@ -89,11 +97,11 @@ def _dissipation_device(prim, mu, T_ref, sutherland, rho_ref, L_box):
     nz, ny, nx = prim.shape[1:]
     with torch.cuda.device(prim.device):
         L, stream = lbm.lib(), torch.cuda.current_stream().cuda_stream
-        uh = torch.fft.rfftn(prim[1:4], dim=(1, 2, 3)).contiguous()
-        wh = uh.new_empty((4,) + tuple(uh.shape[1:]))
-        lbm.check(L.lbm_spectral_curl_div(uh.data_ptr(), wh.data_ptr(), nx, ny, nz,
+        zh, ch = _packed_spectra(prim[1:4])
+        wh = zh.new_empty((2, nz, ny, nx))
+        lbm.check(L.lbm_spectral_curl_div(zh.data_ptr(), ch.data_ptr(), wh.data_ptr(), nx, ny, nz,
                                           2 * math.pi / L_box, stream))
-        w = torch.fft.irfftn(wh, s=(nz, ny, nx), dim=(1, 2, 3), norm="forward").contiguous()
+        w = torch.fft.ifftn(wh, dim=(1, 2, 3), norm="forward").contiguous()
         T = prim[4].contiguous()
         out = torch.empty(_DOUBLES, dtype=torch.float64, device=prim.device)
         lbm.check(L.lbm_spectral_dissipation(w.data_ptr(), T.data_ptr(), nx * ny * nz, mu, T_ref,
@@ -112,10 +120,10 @@ def energy_spectrum(u, L_box=2 * math.pi):
         shells = L.lbm_spectral_shell_count(nx, ny, nz)
         if shells <= _MOST_SHELLS:
             with torch.cuda.device(u.device):
-                uh = torch.fft.rfftn(u, dim=(1, 2, 3)).contiguous()
+                zh, ch = _packed_spectra(u)
                 e = torch.zeros(shells, dtype=u.dtype, device=u.device)
-                lbm.check(L.lbm_spectral_shells(uh.data_ptr(), nx, ny, nz, e.data_ptr(), shells,
-                                                torch.cuda.current_stream().cuda_stream))
+                lbm.check(L.lbm_spectral_shells(zh.data_ptr(), ch.data_ptr(), nx, ny, nz, e.data_ptr(),
+                                                shells, torch.cuda.current_stream().cuda_stream))
                 return torch.arange(shells, device=u.device), e
     dt = u.dtype
     kx = _k_full(nx, L_box, u.device, dt).view(1, 1, nx)
