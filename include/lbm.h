@@ -151,8 +151,8 @@ typedef struct {
                                memory by bulk asynchronous copies, a persistent grid of
                                4-warp blocks: 2 stages per warp with <= 170 registers (2),
                                2 stages with <= 128 (3), 3 stages with <= 170 (4) */
-  int prefetch_tiles;       /* L2 prefetch distance of variants 0 and 1 on whole-tile rows
-                               (see lbm_set_prefetch); 0 = off */
+  int prefetch_tiles;       /* L2 prefetch distance of variants 0 and 1 (see
+                               lbm_set_prefetch); 0 = off */
   int device;               /* CUDA device ordinal the handle is bound to (see lbm_create) */
 } lbm_info_t;
 
@@ -341,8 +341,7 @@ lbm_status lbm_load(lbm_handle* h, const char* path);
 /* ---- tuning ------------------------------------------------------------------- */
 
 /* Times the step kernel for each candidate form (variants 0 and 1 at blocks of 64
- * and 128 threads, each with L2 prefetch distances 0, 512, 1024 and 2048 tiles on
- * whole-tile rows: at most 16 candidates; the staged variants 2-4, measured slower
+ * and 128 threads, each with L2 prefetch distances 0, 512, 1024 and 2048 tiles: at most 16 candidates; the staged variants 2-4, measured slower
  * everywhere, only through lbm_set_kernel_config) on whole step pairs with CUDA events
  * on the handle's stream, and keeps the fastest in the handle; returns it in *out if
  * out != NULL. Needs an initialised state
@@ -362,13 +361,11 @@ lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out);
  * until a re-init. */
 lbm_status lbm_set_kernel_config(lbm_handle* h, int block_x, int variant);
 
-/* Sets the L2 prefetch distance of the plain step kernel (variants 0 and 1) on
- * domains of whole 32-cell tile rows (periodic x, nx a multiple of 32): the warp
+/* Sets the L2 prefetch distance of the plain step kernel (variants 0 and 1): the warp
  * updating tile t first asks L2, with one bulk prefetch per slot run, for the slot
  * blocks that the warp on tile t + tiles will read, so that warp's loads meet L2
  * instead of DRAM (an implementation choice; the paper has no counterpart). 0 turns
- * it off; held-x domains, other row lengths and the staged and batched forms ignore
- * it. The default is 1024 tiles for 16-bit storage and 0 for FP32; lbm_autotune
+ * it off; the staged and batched forms ignore it. The default is 1024 tiles for 16-bit storage and 0 for FP32; lbm_autotune
  * chooses among 0, 512, 1024 and 2048. Populations are bit-identical with any
  * distance. LBM_E_INVAL for tiles < 0 or > 2^20 or a NULL handle. */
 lbm_status lbm_set_prefetch(lbm_handle* h, int tiles);

@@ -984,13 +984,10 @@ lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out) {
     int variant, block, prefetch;
   };
   std::vector<Cand> cands;
-  // The L2 prefetch applies to the plain forms on whole-tile rows only.
-  const bool rows = h->P.bc_x == 0 && h->P.nx % 32 == 0;
   for (int v : {0, 1})
     for (int b : {64, 128})
       if (b <= 32 * ((h->P.nx + 31) / 32) || b == 64)
-        for (int pf : {0, 512, 1024, 2048})
-          if (pf == 0 || rows) cands.push_back({v, b, pf});
+        for (int pf : {0, 512, 1024, 2048}) cands.push_back({v, b, pf});
   // The staged forms (variants 2-4) are not candidates: measured slower than the plain
   // forms at every size and storage type (their shared-memory pipeline costs more
   // instructions per cell than it saves in latency, and the L2 prefetch hides the

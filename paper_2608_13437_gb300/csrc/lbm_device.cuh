@@ -48,7 +48,7 @@ struct DomainConst {
   float scale[kF], inv_scale[kF];
   int sutherland, sensor_mode, collide;
   int sround;         // 16-bit storage rounds stochastically (1) or to nearest (0)
-  int pf_tiles;       // L2 prefetch distance of the plain step kernel on whole-tile rows (0: off)
+  int pf_tiles;       // L2 prefetch distance of the plain step kernel (0: off)
   int eso;            // storage map: 0 AA pattern, 1 esoteric twist (slots 2, 4, 6 shifted)
   double dx64;        // dx in FP64 (the diagnostics' gradient pass takes 1/dx from it)
   unsigned* check;    // checked builds: count of population addresses found outside the buffer

@@ -21,8 +21,15 @@ __device__ __forceinline__ void cell_xyz(const DomainConst& P, long long cell, i
   z = (int)zz;
 }
 
-// Fused step: one launch per time step, grid (ceil(nx/block_x), ny, nz), block_x in
-// {32, 64, 96, 128}; variant selects the register budget (0: 170, 1: 128 registers).
+// Grid of the step kernels: rows of whole tiles (periodic x, nx a multiple of 32) take
+// (ceil(nx/block_x), ny, nz) blocks, any other domain its tiles in index order.
+inline dim3 step_grid(const DomainConst& P, int block_x) {
+  if (P.bc_x == 0 && P.nx % kTile == 0)
+    return dim3((P.nx + block_x - 1) / block_x, P.ny, P.nz);
+  return dim3((unsigned)((P.ntile * kTile + block_x - 1) / block_x));
+}
+
+// Fused step: one launch per time step, grid step_grid, block_x in {32, 64, 96, 128}; variant selects the register budget (0: 170, 1: 128 registers).
 cudaError_t launch_step_f32(const DomainConst& P, int parity, void* pop, const float* ghost,
                             unsigned* flag, int block_x, int variant, cudaStream_t s);
 cudaError_t launch_step_f16(const DomainConst& P, int parity, void* pop, const float* ghost,
@@ -71,7 +78,8 @@ cudaError_t launch_step_diag_bf16(const DomainConst& P, int parity, void* pop, c
                                   cudaStream_t s);
 constexpr int kDiagRecFloats = 17;  // words of one warp record
 inline long long step_diag_record_count(const DomainConst& P, int block_x) {
-  return (long long)((P.nx + block_x - 1) / block_x) * P.ny * P.nz * (block_x / 32);
+  const dim3 g = step_grid(P, block_x);
+  return (long long)g.x * g.y * g.z * (block_x / 32);
 }
 
 // Several steps of a small domain in one cooperative launch, the populations in registers

@@ -22,16 +22,23 @@ __global__ void __launch_bounds__(128, 3) k_step_diag(const DomainConst P, S* __
                                                       unsigned* __restrict__ flag,
                                                       float* __restrict__ ufield,
                                                       float* __restrict__ rec) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  // x of a row's cell, or the linear cell index (see k_step)
+  const long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   DiagAcc acc;
   diag_zero(acc);
   const int lane = threadIdx.x & (kTile - 1);
+  if constexpr (!ROWS) {
+    if (P.pf_tiles > 0 && lane == 0 && x < P.ncell)
+      prefetch_future_linear<PARITY, S>(P, pop, x / kTile);
+  }
   // no early return: every lane takes part in the warp reduction
-  if (ROWS ? (x - lane < P.nx) : (x < P.nx)) {
+  if (ROWS ? (x - lane < P.nx) : (x < P.ncell)) {
     float d[kF][kQ];
     CellDiag cd;
+    long long cell;
     if constexpr (ROWS) {
-      const WarpTiles T = warp_tiles(P, x - lane, blockIdx.y, blockIdx.z);
+      const WarpTiles T = warp_tiles(P, (int)x - lane, blockIdx.y, blockIdx.z);
+      cell = T.t * kTile + lane;
       if (P.pf_tiles > 0 && lane == 0) prefetch_future<PARITY, S, ESO>(P, pop, T.t);
       load_cell_rows<PARITY, S, ESO>(P, pop, T, lane, d);
       if (P.collide) {
@@ -43,7 +50,10 @@ __global__ void __launch_bounds__(128, 3) k_step_diag(const DomainConst P, S* __
       }
       store_cell_rows<PARITY, S, SR, ESO>(P, pop, T, lane, d);
     } else {
-      const CellIndex c = make_index(P, x, blockIdx.y, blockIdx.z);
+      int cx, cy, cz;
+      tile_xyz(P, x / kTile, lane, cx, cy, cz);
+      const CellIndex c = make_index(P, cx, cy, cz);
+      cell = x;
       load_cell<PARITY, HELD, S>(P, pop, ghost, c, d);
       if (P.collide) {
         const float probe = collide_cell<false, true>(P, d, nullptr, &cd);
@@ -56,7 +66,6 @@ __global__ void __launch_bounds__(128, 3) k_step_diag(const DomainConst P, S* __
     }
     diag_add_cell(P, cd, acc);
     const long long n = P.ncell;
-    const long long cell = x + (long long)P.nx * (blockIdx.y + (long long)P.ny * blockIdx.z);
     ufield[cell] = cd.u[0];
     ufield[n + cell] = cd.u[1];
     ufield[2 * n + cell] = cd.u[2];
@@ -91,7 +100,7 @@ cudaError_t launch_step_diag_t(const DomainConst& P, int parity, void* pop, cons
                                cudaStream_t s) {
   if (block_x < 32 || block_x > 128 || (block_x & 31)) return cudaErrorInvalidConfiguration;
   const dim3 block(block_x);
-  const dim3 grid((P.nx + block_x - 1) / block_x, P.ny, P.nz);
+  const dim3 grid = step_grid(P, block_x);
   S* p = static_cast<S*>(pop);
   if constexpr (!std::is_same<S, float>::value) {
     if (P.sround) {

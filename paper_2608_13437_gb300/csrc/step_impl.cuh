@@ -94,6 +94,55 @@ __device__ __forceinline__ void prefetch_future(const DomainConst& P, const S* p
   }
 }
 
+// prefetch_future for tiles of any other row length: the same slot blocks of tile w, and
+// the z slots of the tiles that hold the cells a plane from w's first cell (the next
+// warp's tile covers what lies beyond it). The map is P.eso's.
+template <int PARITY, typename S>
+__device__ __forceinline__ void prefetch_future_linear(const DomainConst& P, const S* pop, long long t) {
+  const long long w = t + P.pf_tiles;
+  if (w >= P.ntile) return;
+  constexpr unsigned kSlotBytes = kSlotElems * sizeof(S);
+  const long long first = w * kTile, nxy = (long long)P.nx * P.ny;
+  const long long up = first + nxy < P.ncell ? first + nxy : first + nxy - P.ncell;
+  const S* const own = pop + w * kTileElems;
+  const S* const zp = pop + (up / kTile) * kTileElems;
+  if (P.eso) {
+    l2_prefetch(own, (PARITY ? 5 : 6) * kSlotBytes);
+    if (PARITY) l2_prefetch(own + 6 * kSlotElems, kSlotBytes);
+    l2_prefetch(zp + (PARITY ? 5 : 6) * kSlotElems, kSlotBytes);
+  } else if (PARITY == 0) {
+    l2_prefetch(own, kQ * kSlotBytes);
+  } else {
+    const long long down = first >= nxy ? first - nxy : first - nxy + P.ncell;
+    l2_prefetch(own, 5 * kSlotBytes);
+    l2_prefetch(pop + (down / kTile) * kTileElems + 6 * kSlotElems, kSlotBytes);
+    l2_prefetch(zp + 5 * kSlotElems, kSlotBytes);
+  }
+}
+
+// (x, y, z) of lane `lane` of tile t: the divisions are warp-uniform (the tile's first
+// cell), the lane carries x past the row end.
+__device__ __forceinline__ void tile_xyz(const DomainConst& P, long long t, int lane, int& x, int& y,
+                                         int& z) {
+  cell_xyz(P, t * kTile, x, y, z);
+  x += lane;
+  if (P.nx >= kTile) {  // at most one row end in a tile
+    if (x >= P.nx) {
+      x -= P.nx;
+      ++y;
+    }
+  } else {
+    const int rows = x / P.nx;
+    x -= rows * P.nx;
+    y += rows;
+  }
+  if (y >= P.ny) {  // rows shorter than a tile may end several planes
+    const int planes = y / P.ny;
+    y -= planes * P.ny;
+    z += planes;
+  }
+}
+
 // load_cell for whole-tile rows: even steps read slot i of the own cell, odd steps
 // slot opp(i) of cell x - e_i; ESO: the esoteric twist, directions -x, -y, -z from the
 // cell x - e_i (= x + e_x, x + e_y, x + e_z) at both parities, the rest from the own cell.
@@ -148,7 +197,12 @@ __device__ __forceinline__ void store_cell_rows(const DomainConst& P, S* __restr
 
 // MINB = resident 128-thread blocks per SM the register budget is sized for:
 // 3 -> at most 170 registers (no spills), 4 -> at most 128 (a few spilled words).
-// ROWS: whole-tile rows (periodic x, nx a multiple of 32), addressed per warp.
+// ROWS: whole-tile rows (periodic x, nx a multiple of 32), addressed per warp. Other
+// domains take one warp per tile too, over the linear cell index, so that every lane but
+// the last tile's works and the own slots are whole aligned tiles: with a grid of rows,
+// 150 cells to a row filled 150 of 192 lanes and its warps straddled two tiles (BF16
+// 150 x 100 x 60: 60 and 67 us at even and odd steps, HBM's time 52 us), and rows shorter
+// than 32 cells filled a fraction of a warp.
 // SR: stochastic rounding of 16-bit storage.
 // ESO: the esoteric twist on whole-tile rows (the other forms take it from P.eso).
 template <int PARITY, typename S, bool HELD, int MINB, bool ROWS, bool SR = false, bool ESO = false>
@@ -169,9 +223,15 @@ __global__ void __launch_bounds__(128, MINB) k_step(const DomainConst P, S* __re
     }
     store_cell_rows<PARITY, S, SR, ESO>(P, pop, T, lane, d);
   } else {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    if (x >= P.nx) return;
-    const CellIndex c = make_index(P, x, blockIdx.y, blockIdx.z);
+    const long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long t = cell / kTile;
+    if (t >= P.ntile) return;  // whole warps
+    const int lane = threadIdx.x & (kTile - 1);
+    if (P.pf_tiles > 0 && lane == 0) prefetch_future_linear<PARITY, S>(P, pop, t);
+    if (cell >= P.ncell) return;
+    int x, y, z;
+    tile_xyz(P, t, lane, x, y, z);
+    const CellIndex c = make_index(P, x, y, z);
     load_cell<PARITY, HELD, S>(P, pop, ghost, c, d);
     if (P.collide) {
       const float probe = collide_cell<false>(P, d, nullptr);
@@ -217,7 +277,7 @@ cudaError_t launch_step_t(const DomainConst& P, int parity, void* pop, const flo
                           unsigned* flag, int block_x, int variant, cudaStream_t s) {
   if (block_x < 32 || block_x > 128 || (block_x & 31)) return cudaErrorInvalidConfiguration;
   const dim3 block(block_x);
-  const dim3 grid((P.nx + block_x - 1) / block_x, P.ny, P.nz);
+  const dim3 grid = step_grid(P, block_x);
   S* p = static_cast<S*>(pop);
   if (variant) launch_variant<S, 4>(P, parity, p, ghost, flag, grid, block, s);
   else launch_variant<S, 3>(P, parity, p, ghost, flag, grid, block, s);
