@@ -715,7 +715,7 @@ lbm_status lbm_moments(lbm_handle* h, int which, void* dst, int dst_on_device, i
     if (e != cudaSuccess) return fail(LBM_E_CUDA, "moments failed: %s", cudaGetErrorString(e));
     return LBM_OK;
   }
-  long long chunk = (long long)(kStageBytes / (es * nf));
+  long long chunk = (long long)(kStageBytes / (es * nf)) / kTile * kTile;  // whole tiles
   if (chunk > h->ncell) chunk = h->ncell;
   lbm_status st = ensure_stage(h);
   if (st != LBM_OK) return st;

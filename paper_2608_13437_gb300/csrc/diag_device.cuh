@@ -38,6 +38,19 @@ __device__ __forceinline__ void ff_merge(FF& a, const FF& b) {
   a.lo = __fsub_rn(e, __fsub_rn(a.hi, s));
 }
 
+// Two float-float accumulators in packed pairs: ff_add of both halves (sums and
+// differences only, so every half rounds as the scalar code does).
+struct FF2 {
+  F2 hi, lo;
+};
+__device__ __forceinline__ void ff_add2(FF2& a, F2 x) {
+  const F2 s = add2(a.hi, x);
+  const F2 bp = sub2(s, a.hi);
+  const F2 e = add2(sub2(a.hi, sub2(s, bp)), sub2(x, bp));
+  a.hi = s;
+  a.lo = add2(a.lo, e);
+}
+
 __device__ __forceinline__ double ff_value(const FF& a) { return (double)a.hi + (double)a.lo; }
 
 // Sums: 0 rho deviations, 1-3 momentum, 4 E deviations, 5 rho |u|^2 / 2.

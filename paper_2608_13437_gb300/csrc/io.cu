@@ -4,6 +4,7 @@
 // raw slot planes.
 #include "diag_device.cuh"
 #include "lbm_internal.h"
+#include "step_impl.cuh"
 
 namespace lbm {
 
@@ -21,23 +22,31 @@ __device__ __forceinline__ double read_dev64(const DomainConst& P, const S* pop,
   return Codec<S>::dec64(pop[read_pos(P, c, parity, k, i)], (double)P.scale[k]);
 }
 
-// Moments of cells [c0, c0 + cnt) through the AA read map of the step's parity, from
-// the step's own loads and FP32 decode. LBM_MOM_Q: per field a float-float sum of the
-// seven populations and the reference (two-sum, about 48 significant bits), widened to
-// the output type. LBM_MOM_PRIM: the primitives exactly as the step computes them (its
-// FP32 sums and closure). No FP64 arithmetic: FP64 here is only an output format.
-template <typename S, int PARITY, bool HELD>
-__global__ void k_moments(const DomainConst P, const S* __restrict__ pop,
-                          const float* __restrict__ ghost, int which, void* out, int out_f64,
-                          long long c0, long long cnt) {
-  for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < cnt;
-       r += (long long)gridDim.x * blockDim.x) {
-    const long long cell = c0 + r;
-    int x, y, z;
-    decompose(P, cell, x, y, z);
-    const CellIndex c = make_index(P, x, y, z);
+// Moments of cells [c0, c0 + cnt) (c0 a multiple of 32) through the AA read map of the
+// step's parity, from the step's own loads and FP32 decode. LBM_MOM_Q: per field a
+// float-float sum of the seven populations and the reference (two-sum, about 48
+// significant bits), widened to the output type. LBM_MOM_PRIM: the primitives exactly as
+// the step computes them (its FP32 sums and closure). No FP64 arithmetic: FP64 here is
+// only an output format.
+// One warp per tile. 16-bit storage is bound by issue here as much as by HBM: the
+// float-float sums go two fields at a time (packed), whole-tile rows take the step's
+// warp-uniform addressing, and 128 registers leave 16 warps an SM (256^3 FP16, Q: 726 us at
+// even and 890 at odd parity with the general index maps and 12 warps, 649 and 680 now;
+// HBM's time for its 4.2 GB is 626. FP32 was at HBM's time and stays there). An L2 prefetch
+// of the tile a warp takes next, with a grid of resident blocks, was slower (744-860).
+constexpr int kMomThreads = 128, kMomBlocks = 4;  // 128 registers a thread
+template <typename S, int PARITY, bool HELD, bool ROWS, bool ESO>
+__global__ void __launch_bounds__(kMomThreads, kMomBlocks)
+    k_moments(const DomainConst P, const S* __restrict__ pop, const float* __restrict__ ghost, int which,
+              void* out, int out_f64, long long c0, long long cnt) {
+  const int lane = threadIdx.x & (kTile - 1);
+  const long long warps = (long long)gridDim.x * (kMomThreads / kTile);
+  const long long tiles = (cnt + kTile - 1) / kTile, t0 = c0 / kTile;
+  for (long long w = blockIdx.x * (long long)(kMomThreads / kTile) + threadIdx.x / kTile; w < tiles; w += warps) {
+    const long long r = w * kTile + lane;
+    if (r >= cnt) continue;
     float d[kF][kQ];
-    load_cell<PARITY, HELD, S>(P, pop, ghost, c, d);
+    load_tile_cell<PARITY, HELD, ROWS, ESO, S>(P, pop, ghost, t0 + w, lane, d);
     if (which == 1) {
       float Q[kF];
 #pragma unroll
@@ -59,14 +68,21 @@ __global__ void k_moments(const DomainConst P, const S* __restrict__ pop,
       }
     } else {
 #pragma unroll
-      for (int k = 0; k < kF; ++k) {
-        FF a = {d[k][0], 0.0f};
+      for (int k = 0; k < kF; k += 2) {
+        FF2 a = {pack2(d[k][0], d[k + 1][0]), pack2(0.0f, 0.0f)};
 #pragma unroll
-        for (int i = 1; i < kQ; ++i) ff_add(a, d[k][i]);
-        if (k == 0) ff_add(a, P.rho_ref);
-        if (k == 4) ff_add(a, P.E_ref);
-        if (out_f64) static_cast<double*>(out)[(long long)k * cnt + r] = ff_value(a);
-        else static_cast<float*>(out)[(long long)k * cnt + r] = add(a.hi, a.lo);
+        for (int i = 1; i < kQ; ++i) ff_add2(a, pack2(d[k][i], d[k + 1][i]));
+        if (k == 0) ff_add2(a, pack2(P.rho_ref, -0.0f));
+        if (k == 4) ff_add2(a, pack2(P.E_ref, -0.0f));
+        FF v[2];
+        unpack2(a.hi, v[0].hi, v[1].hi);
+        unpack2(a.lo, v[0].lo, v[1].lo);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const long long at = (long long)(k + j) * cnt + r;
+          if (out_f64) static_cast<double*>(out)[at] = ff_value(v[j]);
+          else static_cast<float*>(out)[at] = add(v[j].hi, v[j].lo);
+        }
       }
     }
   }
@@ -74,15 +90,16 @@ __global__ void k_moments(const DomainConst P, const S* __restrict__ pop,
 
 template <typename S>
 void launch_moments_t(const DomainConst& P, int parity, const S* pop, const float* ghost, int which,
-                      void* out, int out_f64, long long c0, long long cnt, int grid, int block,
-                      cudaStream_t s) {
-  if (P.bc_x) {
-    if (parity) k_moments<S, 1, true><<<grid, block, 0, s>>>(P, pop, ghost, which, out, out_f64, c0, cnt);
-    else k_moments<S, 0, true><<<grid, block, 0, s>>>(P, pop, ghost, which, out, out_f64, c0, cnt);
-  } else {
-    if (parity) k_moments<S, 1, false><<<grid, block, 0, s>>>(P, pop, ghost, which, out, out_f64, c0, cnt);
-    else k_moments<S, 0, false><<<grid, block, 0, s>>>(P, pop, ghost, which, out, out_f64, c0, cnt);
-  }
+                      void* out, int out_f64, long long c0, long long cnt, cudaStream_t s) {
+  const int block = kMomThreads;
+  const long long need = (cnt + kMomThreads - 1) / kMomThreads;
+  const long long most = (long long)sm_count() * 32;
+  const unsigned grid = (unsigned)(need < most ? need : most);
+  with_tile_form(P, parity, [&](auto f) {
+    using F = decltype(f);
+    k_moments<S, F::parity, F::held, F::rows, F::eso>
+        <<<grid, block, 0, s>>>(P, pop, ghost, which, out, out_f64, c0, cnt);
+  });
 }
 
 template <typename S>
@@ -189,11 +206,10 @@ int grid_for(long long n, int block) {
 cudaError_t launch_moments(const DomainConst& P, int store, int parity, const void* pop,
                            const float* ghost, int which, void* out, int out_f64, long long c0,
                            long long cnt, cudaStream_t s) {
-  const int block = 128, grid = grid_for(cnt, block);
   switch (store) {
-    case 0: launch_moments_t(P, parity, (const float*)pop, ghost, which, out, out_f64, c0, cnt, grid, block, s); break;
-    case 1: launch_moments_t(P, parity, (const __half*)pop, ghost, which, out, out_f64, c0, cnt, grid, block, s); break;
-    default: launch_moments_t(P, parity, (const __nv_bfloat16*)pop, ghost, which, out, out_f64, c0, cnt, grid, block, s); break;
+    case 0: launch_moments_t(P, parity, (const float*)pop, ghost, which, out, out_f64, c0, cnt, s); break;
+    case 1: launch_moments_t(P, parity, (const __half*)pop, ghost, which, out, out_f64, c0, cnt, s); break;
+    default: launch_moments_t(P, parity, (const __nv_bfloat16*)pop, ghost, which, out, out_f64, c0, cnt, s); break;
   }
   return cudaGetLastError();
 }

@@ -364,6 +364,11 @@ __device__ __forceinline__ float ghost_value(const DomainConst& P, const float* 
   return ghost[((long long)side * kF + k) * planes + c.plane];
 }
 
+// Bulk prefetch of `bytes` (a multiple of 16, 16-byte aligned) into L2.
+__device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // Loads the 98 decoded deviations of this cell for a step of the given parity:
 // per direction i the source cell and slot of the AA map (or the esoteric twist), then
 // 4 + 4 + 4 + 2 fields.

@@ -21,6 +21,29 @@ __device__ __forceinline__ void cell_xyz(const DomainConst& P, long long cell, i
   z = (int)zz;
 }
 
+// (x, y, z) of lane `lane` of tile t: the divisions are warp-uniform (the tile's first
+// cell), the lane carries x past the row end.
+__device__ __forceinline__ void tile_xyz(const DomainConst& P, long long t, int lane, int& x, int& y,
+                                         int& z) {
+  cell_xyz(P, t * kTile, x, y, z);
+  x += lane;
+  if (P.nx >= kTile) {  // at most one row end in a tile
+    if (x >= P.nx) {
+      x -= P.nx;
+      ++y;
+    }
+  } else {
+    const int rows = x / P.nx;
+    x -= rows * P.nx;
+    y += rows;
+  }
+  if (y >= P.ny) {  // rows shorter than a tile may end several planes
+    const int planes = y / P.ny;
+    y -= planes * P.ny;
+    z += planes;
+  }
+}
+
 // Grid of the step kernels: rows of whole tiles (periodic x, nx a multiple of 32) take
 // (ceil(nx/block_x), ny, nz) blocks, any other domain its tiles in index order.
 inline dim3 step_grid(const DomainConst& P, int block_x) {
@@ -101,6 +124,9 @@ size_t resident_inbox_bytes(const ResidentPlan& R, int store);
 cudaError_t launch_resident(const DomainConst& P, const ResidentPlan& R, int store, int parity,
                             void* pop, const float* ghost, unsigned* flag, void* inbox,
                             unsigned* epochs, int steps, cudaStream_t s);
+
+// SMs of the current device (looked up once per device).
+int sm_count();
 
 // Initial states (init.cu). kind: 0 TGV, 1 Riemann, 2 caller fields (rho, u, p),
 // 3 caller zeroth moments (14 fields). Host-computed FP32 constants; the device works

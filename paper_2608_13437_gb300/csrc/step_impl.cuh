@@ -50,11 +50,6 @@ __device__ __forceinline__ void link_tile(const WarpTiles& T, int i, int toward,
   }
 }
 
-// Bulk prefetch of `bytes` (a multiple of 16, 16-byte aligned) into L2.
-__device__ __forceinline__ void l2_prefetch(const void* p, unsigned bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 // Whole-tile rows: tiles are processed roughly in index order, so the warp on tile t
 // asks L2 for the slot blocks that the warp on tile w = t + P.pf_tiles will read, and
 // that warp later finds them in L2 instead of waiting on DRAM. Even steps read the 7
@@ -120,29 +115,6 @@ __device__ __forceinline__ void prefetch_future_linear(const DomainConst& P, con
   }
 }
 
-// (x, y, z) of lane `lane` of tile t: the divisions are warp-uniform (the tile's first
-// cell), the lane carries x past the row end.
-__device__ __forceinline__ void tile_xyz(const DomainConst& P, long long t, int lane, int& x, int& y,
-                                         int& z) {
-  cell_xyz(P, t * kTile, x, y, z);
-  x += lane;
-  if (P.nx >= kTile) {  // at most one row end in a tile
-    if (x >= P.nx) {
-      x -= P.nx;
-      ++y;
-    }
-  } else {
-    const int rows = x / P.nx;
-    x -= rows * P.nx;
-    y += rows;
-  }
-  if (y >= P.ny) {  // rows shorter than a tile may end several planes
-    const int planes = y / P.ny;
-    y -= planes * P.ny;
-    z += planes;
-  }
-}
-
 // load_cell for whole-tile rows: even steps read slot i of the own cell, odd steps
 // slot opp(i) of cell x - e_i; ESO: the esoteric twist, directions -x, -y, -z from the
 // cell x - e_i (= x + e_x, x + e_y, x + e_z) at both parities, the rest from the own cell.
@@ -192,6 +164,48 @@ __device__ __forceinline__ void store_cell_rows(const DomainConst& P, S* __restr
     if (ESO ? (i == 1 || i == 3 || i == 5) : (PARITY && i > 0)) link_tile(T, i, +1, lane, tile, ln);
     if (!LBM_CHECK(P, tile >= 0 && tile < P.ntile)) continue;
     store_dir<S>(P, pop + tile * kTileElems, PARITY ? i : opp(i), ln, d, i, SR ? &dz : nullptr);
+  }
+}
+
+// The decoded deviations of lane `lane`'s cell of tile t, for kernels that walk the tiles
+// in index order (outputs and diagnostics): whole-tile rows through the warp-uniform
+// addressing of the step (about 60 instructions less per cell than the general index
+// maps, which counts where 16-bit decoding makes them issue-bound), the others through
+// load_cell.
+template <int PARITY, bool HELD, bool ROWS, bool ESO, typename S>
+__device__ __forceinline__ void load_tile_cell(const DomainConst& P, const S* __restrict__ pop,
+                                               const float* __restrict__ ghost, long long t, int lane,
+                                               float (&d)[kF][kQ]) {
+  int x, y, z;
+  if constexpr (ROWS) {
+    cell_xyz(P, t * kTile, x, y, z);
+    load_cell_rows<PARITY, S, ESO>(P, pop, warp_tiles(P, x, y, z), lane, d);
+  } else {
+    tile_xyz(P, t, lane, x, y, z);
+    load_cell<PARITY, HELD, S>(P, pop, ghost, make_index(P, x, y, z), d);
+  }
+}
+
+// Calls f with the compile-time form of load_tile_cell that suits the domain.
+template <int PARITY, bool HELD, bool ROWS, bool ESO>
+struct TileForm {
+  static constexpr int parity = PARITY;
+  static constexpr bool held = HELD, rows = ROWS, eso = ESO;
+};
+template <typename F>
+void with_tile_form(const DomainConst& P, int parity, F&& f) {
+  if (P.bc_x) {
+    if (parity) f(TileForm<1, true, false, false>{});
+    else f(TileForm<0, true, false, false>{});
+  } else if (P.nx % kTile == 0 && P.eso) {
+    if (parity) f(TileForm<1, false, true, true>{});
+    else f(TileForm<0, false, true, true>{});
+  } else if (P.nx % kTile == 0) {
+    if (parity) f(TileForm<1, false, true, false>{});
+    else f(TileForm<0, false, true, false>{});
+  } else {
+    if (parity) f(TileForm<1, false, false, false>{});
+    else f(TileForm<0, false, false, false>{});
   }
 }
 
