@@ -274,7 +274,7 @@ lbm_status lbm_synchronize(lbm_handle* h);
  * float-float sum (about 48 significant bits) of the seven populations and the
  * reference; the primitives are exactly the step's own (its FP32 sums and closure).
  * Synchronises when dst is on the host (through a device staging buffer the handle
- * keeps, 256 MB, allocated on first use). */
+ * keeps, of at most 256 MB, allocated on first use). */
 lbm_status lbm_moments(lbm_handle* h, int which, void* dst, int dst_on_device, int dtype);
 
 /* Sensor of the current state, [3][z][y][x]: theta = div u (physical units),

@@ -9,6 +9,8 @@
 #include <vector>
 
 #include "api_common.h"
+#include "host_pages.h"
+#include "lbm_arrays.h"
 
 using namespace lbm;
 
@@ -183,7 +185,8 @@ struct lbm_handle {
   float* wrec = nullptr;       // per-warp records of the diagnostic step
   long long wrec_n = 0;
   double* hdiag = nullptr;     // pinned host copy of dout and the flag
-  void* stage = nullptr;       // device staging for host-side outputs (kStageBytes)
+  void* stage = nullptr;       // device staging for transfers to and from host memory
+  size_t stage_bytes = 0;
   cudaEvent_t ev_diag = nullptr;
   // resident form (step_resident.cu): bricks, their inboxes and step counts (one block)
   ResidentPlan res;
@@ -564,16 +567,20 @@ static void* mapped_host(const void* p, size_t align) {
   return a.devicePointer;
 }
 
-static lbm_status init_from_fields(lbm_handle* h, const void* fields, int src_on_device, int dtype,
-                                   int kind, int nfield) {
+// arrays: nfield separate host arrays in place of one at `fields` (NULL: one array).
+static lbm_status init_from_fields(lbm_handle* h, const void* fields, const void* const* arrays,
+                                   int src_on_device, int dtype, int kind, int nfield) {
   Range range_("lbm_init_fields");
-  if (!h || !fields) return fail(LBM_E_INVAL, "NULL argument");
+  if (!h || (!fields && !arrays)) return fail(LBM_E_INVAL, "NULL argument");
+  if (arrays)
+    for (int j = 0; j < nfield; ++j)
+      if (!arrays[j]) return fail(LBM_E_INVAL, "NULL argument");
   LBM_ON_DEVICE(h->device);
   if (dtype != LBM_DT_F32 && dtype != LBM_DT_F64) return fail(LBM_E_INVAL, "dtype must be F32 or F64");
   const size_t bytes = (size_t)nfield * h->ncell * (dtype == LBM_DT_F64 ? 8 : 4);
   void* dev = const_cast<void*>(fields);
   void* tmp = nullptr;
-  void* mapped = src_on_device ? nullptr : mapped_host(fields, dtype == LBM_DT_F64 ? 8 : 4);
+  void* mapped = src_on_device || arrays ? nullptr : mapped_host(fields, dtype == LBM_DT_F64 ? 8 : 4);
   if (mapped) {
     dev = mapped;  // page-locked: the kernels read it directly
   } else if (!src_on_device) {
@@ -581,8 +588,13 @@ static lbm_status init_from_fields(lbm_handle* h, const void* fields, int src_on
       cudaGetLastError();
       return fail(LBM_E_NOMEM, "cudaMalloc of %zu staging bytes failed", bytes);
     }
-    cudaError_t e = cudaMemcpyAsync(tmp, fields, bytes, cudaMemcpyHostToDevice, h->stream);
+    cudaError_t e = cudaSuccess;
+    const size_t part = arrays ? bytes / nfield : bytes;
+    for (int j = 0; j < (arrays ? nfield : 1) && e == cudaSuccess; ++j)
+      e = cudaMemcpyAsync(static_cast<char*>(tmp) + j * part, arrays ? arrays[j] : fields, part,
+                          cudaMemcpyHostToDevice, h->stream);
     if (e != cudaSuccess) {
+      cudaStreamSynchronize(h->stream);  // none of the arrays' copies still reads or writes
       cudaFree(tmp);
       return fail(LBM_E_CUDA, "copy of initial fields failed: %s", cudaGetErrorString(e));
     }
@@ -612,11 +624,15 @@ static lbm_status init_from_fields(lbm_handle* h, const void* fields, int src_on
 }
 
 lbm_status lbm_init_fields(lbm_handle* h, const void* fields, int src_on_device, int dtype) {
-  return init_from_fields(h, fields, src_on_device, dtype, 2, 5);
+  return init_from_fields(h, fields, nullptr, src_on_device, dtype, 2, 5);
+}
+
+lbm_status lbm_init_fields_arrays(lbm_handle* h, const void* const fields[5], int dtype) {
+  return init_from_fields(h, nullptr, fields, 0, dtype, 2, 5);
 }
 
 lbm_status lbm_init_state(lbm_handle* h, const void* Q, int src_on_device, int dtype) {
-  return init_from_fields(h, Q, src_on_device, dtype, 3, kF);
+  return init_from_fields(h, Q, nullptr, src_on_device, dtype, 3, kF);
 }
 
 lbm_status lbm_step(lbm_handle* h, int n) {
@@ -682,16 +698,51 @@ lbm_status lbm_synchronize(lbm_handle* h) {
   return LBM_OK;
 }
 
-// The handle's device staging buffer for outputs written to host memory, allocated on
-// first use and kept (no allocation or implicit device synchronisation per call).
-static lbm_status ensure_stage(lbm_handle* h) {
-  if (h->stage) return LBM_OK;
-  if (cudaMalloc(&h->stage, kStageBytes) != cudaSuccess) {
+// The handle's device staging buffer for transfers to and from host memory, allocated on
+// first use and kept (no allocation or implicit device synchronisation per call); at most
+// kStageBytes, replaced by a larger one when a transfer needs it.
+static lbm_status ensure_stage(lbm_handle* h, size_t bytes) {
+  if (h->stage_bytes >= bytes) return LBM_OK;
+  if (h->stage) {
+    cudaStreamSynchronize(h->stream);
+    cudaFree(h->stage);
+  }
+  h->stage = nullptr;
+  h->stage_bytes = 0;
+  if (cudaMalloc(&h->stage, bytes) != cudaSuccess) {
     cudaGetLastError();
     h->stage = nullptr;
     return fail(LBM_E_NOMEM, "staging allocation failed");
   }
+  h->stage_bytes = bytes;
   return LBM_OK;
+}
+
+// Cells per staged piece of rows of cell_bytes in all: whole tiles, at most kStageBytes.
+static long long stage_cells(const lbm_handle* h, size_t cell_bytes) {
+  const long long most = (long long)(kStageBytes / cell_bytes) / kTile * kTile;
+  return most < h->ncell ? most : h->ncell;
+}
+
+// Copies the staged rows [rows][cnt] of cells [c0, c0 + cnt) to the host array [rows][ncell]
+// (or back): one copy when the piece is the whole domain, else one plain copy per row.
+static cudaError_t stage_copy(lbm_handle* h, void* host, int rows, size_t es, long long c0, long long cnt,
+                              bool to_host) {
+  char* hp = static_cast<char*>(host);
+  char* dp = static_cast<char*>(h->stage);
+  if (cnt == h->ncell) {
+    const size_t bytes = (size_t)rows * cnt * es;
+    return to_host ? cudaMemcpyAsync(hp, dp, bytes, cudaMemcpyDeviceToHost, h->stream)
+                   : cudaMemcpyAsync(dp, hp, bytes, cudaMemcpyHostToDevice, h->stream);
+  }
+  cudaError_t e = cudaSuccess;
+  for (int j = 0; j < rows && e == cudaSuccess; ++j) {
+    char* hr = hp + ((size_t)j * h->ncell + c0) * es;
+    char* dr = dp + (size_t)j * cnt * es;
+    e = to_host ? cudaMemcpyAsync(hr, dr, (size_t)cnt * es, cudaMemcpyDeviceToHost, h->stream)
+                : cudaMemcpyAsync(dr, hr, (size_t)cnt * es, cudaMemcpyHostToDevice, h->stream);
+  }
+  return e;
 }
 
 lbm_status lbm_moments(lbm_handle* h, int which, void* dst, int dst_on_device, int dtype) {
@@ -715,20 +766,16 @@ lbm_status lbm_moments(lbm_handle* h, int which, void* dst, int dst_on_device, i
     if (e != cudaSuccess) return fail(LBM_E_CUDA, "moments failed: %s", cudaGetErrorString(e));
     return LBM_OK;
   }
-  long long chunk = (long long)(kStageBytes / (es * nf)) / kTile * kTile;  // whole tiles
-  if (chunk > h->ncell) chunk = h->ncell;
-  lbm_status st = ensure_stage(h);
+  const long long chunk = stage_cells(h, es * nf);
+  lbm_status st = ensure_stage(h, (size_t)chunk * es * nf);
   if (st != LBM_OK) return st;
-  void* tmp = h->stage;
   cudaError_t e = cudaSuccess;
   for (long long c0 = 0; c0 < h->ncell && e == cudaSuccess; c0 += chunk) {
     const long long cnt = (c0 + chunk <= h->ncell) ? chunk : h->ncell - c0;
-    e = launch_moments(h->P, h->prm.store, parity, h->pop, h->ghost, which, tmp,
+    e = launch_moments(h->P, h->prm.store, parity, h->pop, h->ghost, which, h->stage,
                        dtype == LBM_DT_F64, c0, cnt, h->stream);
-    for (int j = 0; j < nf && e == cudaSuccess; ++j)  // one plain copy per field row
-      e = cudaMemcpyAsync(static_cast<char*>(dst) + ((size_t)j * h->ncell + c0) * es,
-                          static_cast<char*>(tmp) + (size_t)j * cnt * es, (size_t)cnt * es,
-                          cudaMemcpyDeviceToHost, h->stream);
+    if (c0 == 0) populate_host_pages(dst, (size_t)nf * h->ncell * es);  // while the kernel runs
+    if (e == cudaSuccess) e = stage_copy(h, dst, nf, es, c0, cnt, true);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return fail(LBM_E_CUDA, "moments failed: %s", cudaGetErrorString(e));
@@ -753,20 +800,16 @@ lbm_status lbm_sensor(lbm_handle* h, void* dst, int dst_on_device, int dtype) {
     if (e != cudaSuccess) return fail(LBM_E_CUDA, "sensor failed: %s", cudaGetErrorString(e));
     return LBM_OK;
   }
-  long long chunk = (long long)(kStageBytes / (es * 3));
-  if (chunk > h->ncell) chunk = h->ncell;
-  lbm_status st = ensure_stage(h);
+  const long long chunk = stage_cells(h, es * 3);
+  lbm_status st = ensure_stage(h, (size_t)chunk * es * 3);
   if (st != LBM_OK) return st;
-  void* tmp = h->stage;
   cudaError_t e = cudaSuccess;
   for (long long c0 = 0; c0 < h->ncell && e == cudaSuccess; c0 += chunk) {
     const long long cnt = (c0 + chunk <= h->ncell) ? chunk : h->ncell - c0;
-    e = launch_sensor(h->P, h->prm.store, parity, h->pop, h->ghost, tmp, dtype == LBM_DT_F64, c0, cnt,
+    e = launch_sensor(h->P, h->prm.store, parity, h->pop, h->ghost, h->stage, dtype == LBM_DT_F64, c0, cnt,
                       h->stream);
-    for (int j = 0; j < 3 && e == cudaSuccess; ++j)
-      e = cudaMemcpyAsync(static_cast<char*>(dst) + ((size_t)j * h->ncell + c0) * es,
-                          static_cast<char*>(tmp) + (size_t)j * cnt * es, (size_t)cnt * es,
-                          cudaMemcpyDeviceToHost, h->stream);
+    if (c0 == 0) populate_host_pages(dst, (size_t)3 * h->ncell * es);
+    if (e == cudaSuccess) e = stage_copy(h, dst, 3, es, c0, cnt, true);
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return fail(LBM_E_CUDA, "sensor failed: %s", cudaGetErrorString(e));
@@ -896,30 +939,34 @@ static lbm_status pop_transfer(lbm_handle* h, void* buf, int on_device, int dtyp
   if (dtype != LBM_DT_F32 && dtype != LBM_DT_F64 && dtype != LBM_DT_NATIVE)
     return fail(LBM_E_INVAL, "bad dtype");
   const size_t es = dtype == LBM_DT_F64 ? 8 : (dtype == LBM_DT_F32 ? 4 : elem_size(h->prm.store));
-  const size_t arr = es * (size_t)h->ncell;
   const int parity = (int)(h->step & 1);
-  void* tmp = nullptr;
-  if (!on_device && cudaMalloc(&tmp, arr) != cudaSuccess) {
-    cudaGetLastError();
-    return fail(LBM_E_NOMEM, "staging allocation failed");
-  }
+  auto move = [&](void* dev, long long c0, long long cnt) {
+    return launch_populations(h->P, h->prm.store, parity, h->pop, h->ghost, dev, dtype, get ? 0 : 1, c0, cnt,
+                              h->stream);
+  };
   cudaError_t e = cudaSuccess;
-  for (int k = 0; k < kF && e == cudaSuccess; ++k)
-    for (int i = 0; i < kQ && e == cudaSuccess; ++i) {
-      char* user = static_cast<char*>(buf) + (size_t)(k * kQ + i) * arr;
-      void* dev = on_device ? (void*)user : tmp;
+  if (on_device) {
+    e = move(buf, 0, h->ncell);
+  } else if (void* m = mapped_host(buf, es)) {  // page-locked: the kernel moves it directly
+    e = move(m, 0, h->ncell);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  } else {
+    const long long chunk = stage_cells(h, es * kP);
+    lbm_status st = ensure_stage(h, (size_t)chunk * es * kP);
+    if (st != LBM_OK) return st;
+    for (long long c0 = 0; c0 < h->ncell && e == cudaSuccess; c0 += chunk) {
+      const long long cnt = (c0 + chunk <= h->ncell) ? chunk : h->ncell - c0;
       if (get) {
-        e = launch_pop_get(h->P, h->prm.store, parity, h->pop, h->ghost, k, i, dev, dtype, h->stream);
-        if (e == cudaSuccess && !on_device)
-          e = cudaMemcpyAsync(user, tmp, arr, cudaMemcpyDeviceToHost, h->stream);
+        e = move(h->stage, c0, cnt);
+        if (c0 == 0) populate_host_pages(buf, es * (size_t)h->ncell * kP);
+        if (e == cudaSuccess) e = stage_copy(h, buf, kP, es, c0, cnt, true);
       } else {
-        if (!on_device) e = cudaMemcpyAsync(tmp, user, arr, cudaMemcpyHostToDevice, h->stream);
-        if (e == cudaSuccess)
-          e = launch_pop_set(h->P, h->prm.store, parity, h->pop, k, i, dev, dtype, h->stream);
+        e = stage_copy(h, buf, kP, es, c0, cnt, false);
+        if (e == cudaSuccess) e = move(h->stage, c0, cnt);
       }
-      if (e == cudaSuccess && !on_device) e = cudaStreamSynchronize(h->stream);
     }
-  if (tmp) cudaFree(tmp);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  }
   if (e != cudaSuccess) return fail(LBM_E_CUDA, "population transfer failed: %s", cudaGetErrorString(e));
   return LBM_OK;
 }

@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "api_common.h"
+#include "host_pages.h"
 #include "step_impl.cuh"
 
 using namespace lbm;
@@ -575,8 +576,10 @@ lbm_status lbm_batch_moments(lbm_batch* b, int domain, int which, void* dst, int
   }
   cudaError_t e = launch_moments(P, b->store, (int)(b->step & 1), domain_pop(b, domain), b->ghost,
                                  which, dev, dtype == LBM_DT_F64, 0, P.ncell, b->stream);
-  if (e == cudaSuccess && !dst_on_device)
+  if (e == cudaSuccess && !dst_on_device) {
+    populate_host_pages(dst, bytes);  // while the kernel runs
     e = cudaMemcpyAsync(dst, dev, bytes, cudaMemcpyDeviceToHost, b->stream);
+  }
   if (e == cudaSuccess && !dst_on_device) e = cudaStreamSynchronize(b->stream);
   if (!dst_on_device) cudaFree(dev);
   if (e != cudaSuccess) return fail(LBM_E_CUDA, "batch moments failed: %s", cudaGetErrorString(e));

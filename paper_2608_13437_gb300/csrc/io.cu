@@ -15,13 +15,6 @@ __device__ __forceinline__ void decompose(const DomainConst& P, long long cell, 
   cell_xyz(P, cell, x, y, z);
 }
 
-template <typename S>
-__device__ __forceinline__ double read_dev64(const DomainConst& P, const S* pop, const float* ghost,
-                                             const CellIndex& c, int parity, int k, int i) {
-  if (from_ghost(P, c, i)) return (double)ghost_value(P, ghost, c, k, i);
-  return Codec<S>::dec64(pop[read_pos(P, c, parity, k, i)], (double)P.scale[k]);
-}
-
 // Moments of cells [c0, c0 + cnt) (c0 a multiple of 32) through the AA read map of the
 // step's parity, from the step's own loads and FP32 decode. LBM_MOM_Q: per field a
 // float-float sum of the seven populations and the reference (two-sum, about 48
@@ -136,45 +129,87 @@ __device__ __forceinline__ double ref_of(const DomainConst& P, int k) {
   return k == 0 ? (double)P.rho_ref : (k == 4 ? (double)P.E_ref : 0.0);
 }
 
-template <typename S>
-__global__ void k_pop_get(const DomainConst P, int parity, const S* __restrict__ pop,
-                          const float* __restrict__ ghost, int k, int i, void* out, int dtype) {
-  for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < P.ncell;
-       cell += (long long)gridDim.x * blockDim.x) {
+// Canonical populations of cells [c0, c0 + cnt) (c0 a multiple of 32), buf[(k, i)][cnt],
+// decoded (dtype F32/F64) or native, out of the state (SET = 0) or into it. One warp per
+// tile moves all 98 arrays: a direction's 14 fields by the layout's vector accesses, the
+// arrays in runs of 32 cells. (One launch per array read or wrote 4 of every 16 bytes of
+// the layout and took 98 x 6 us at 64^3; this is bound by the link or by HBM.)
+// S: storage type, T: the arrays' element type; NATIVE moves the stored bits (S == T), the
+// ghost value encoded like a stored one.
+template <typename S, typename T, bool NATIVE, bool SET>
+__global__ void __launch_bounds__(kMomThreads, kMomBlocks) k_populations(const DomainConst P, int parity,
+                                                             S* __restrict__ pop,
+                                                             const float* __restrict__ ghost,
+                                                             T* __restrict__ buf, long long c0,
+                                                             long long cnt) {
+  using V4 = typename Codec<S>::V4;
+  using V2 = typename Codec<S>::V2;
+  union Fields {  // a direction's 14 fields as the layout's groups
+    struct {
+      V4 v4[3];
+      V2 v2;
+    };
+    S f[kF];
+    __device__ Fields() {}
+  };
+  const int lane = threadIdx.x & (kTile - 1);
+  const long long warps = (long long)gridDim.x * (kMomThreads / kTile);
+  const long long tiles = (cnt + kTile - 1) / kTile, t0 = c0 / kTile;
+  for (long long w = blockIdx.x * (long long)(kMomThreads / kTile) + threadIdx.x / kTile; w < tiles; w += warps) {
+    const long long r = w * kTile + lane;
+    if (r >= cnt) continue;
     int x, y, z;
-    decompose(P, cell, x, y, z);
+    tile_xyz(P, t0 + w, lane, x, y, z);
     const CellIndex c = make_index(P, x, y, z);
-    if (dtype == 2) {  // native bits; the ghost value is encoded like a stored one
-      S g = from_ghost(P, c, i) ? Codec<S>::enc(ghost_value(P, ghost, c, k, i), P.inv_scale[k])
-                                : pop[read_pos(P, c, parity, k, i)];
-      static_cast<S*>(out)[cell] = g;
-      continue;
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+      const bool held = from_ghost(P, c, i);
+      if (SET && held) continue;  // held ends keep the ghost inflow
+      const long long cell = src_cell(P, c, parity, i);
+      if (!LBM_CHECK(P, cell >= 0 && cell < P.ntile * kTile)) continue;
+      S* const base = pop + tile_start(cell);
+      const int slot = parity ? opp(i) : i, ln = (int)(cell & (kTile - 1));
+      Fields u;
+      if (!SET && !held) {
+#pragma unroll
+        for (int g = 0; g < 3; ++g) u.v4[g] = *reinterpret_cast<const V4*>(base + group_offset(slot, g, ln));
+        u.v2 = *reinterpret_cast<const V2*>(base + group_offset(slot, 3, ln));
+      }
+#pragma unroll
+      for (int k = 0; k < kF; ++k) {
+        T* const at = buf + (long long)(k * kQ + i) * cnt + r;
+        if constexpr (SET) {
+          if constexpr (NATIVE) u.f[k] = *at;
+          else u.f[k] = Codec<S>::enc((float)((double)*at - weight(i) * ref_of(P, k)), P.inv_scale[k]);
+        } else if constexpr (NATIVE) {
+          *at = held ? Codec<S>::enc(ghost_value(P, ghost, c, k, i), P.inv_scale[k]) : u.f[k];
+        } else {
+          const double dev = held ? (double)ghost_value(P, ghost, c, k, i)
+                                  : Codec<S>::dec64(u.f[k], (double)P.scale[k]);
+          *at = (T)(weight(i) * ref_of(P, k) + dev);
+        }
+      }
+      if constexpr (SET) {
+#pragma unroll
+        for (int g = 0; g < 3; ++g) *reinterpret_cast<V4*>(base + group_offset(slot, g, ln)) = u.v4[g];
+        *reinterpret_cast<V2*>(base + group_offset(slot, 3, ln)) = u.v2;
+      }
     }
-    const double f = weight(i) * ref_of(P, k) + read_dev64(P, pop, ghost, c, parity, k, i);
-    if (dtype == 1) static_cast<double*>(out)[cell] = f;
-    else static_cast<float*>(out)[cell] = (float)f;
   }
 }
 
-template <typename S>
-__global__ void k_pop_set(const DomainConst P, int parity, S* __restrict__ pop, int k, int i,
-                          const void* in, int dtype) {
-  for (long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x; cell < P.ncell;
-       cell += (long long)gridDim.x * blockDim.x) {
-    int x, y, z;
-    decompose(P, cell, x, y, z);
-    const CellIndex c = make_index(P, x, y, z);
-    if (from_ghost(P, c, i)) continue;  // held ends keep the ghost inflow
-    S g;
-    if (dtype == 2) {
-      g = static_cast<const S*>(in)[cell];
-    } else {
-      const double f = dtype == 1 ? static_cast<const double*>(in)[cell]
-                                  : (double)static_cast<const float*>(in)[cell];
-      g = Codec<S>::enc((float)(f - weight(i) * ref_of(P, k)), P.inv_scale[k]);
-    }
-    pop[read_pos(P, c, parity, k, i)] = g;
-  }
+template <typename S, bool SET>
+void launch_populations_t(const DomainConst& P, int parity, void* pop, const float* ghost, void* buf,
+                          int dtype, long long c0, long long cnt, cudaStream_t s) {
+  const long long need = (cnt + kMomThreads - 1) / kMomThreads, most = (long long)sm_count() * 32;
+  const unsigned grid = (unsigned)(need < most ? need : most);
+  S* p = static_cast<S*>(pop);
+  if (dtype == 2)
+    k_populations<S, S, true, SET><<<grid, kMomThreads, 0, s>>>(P, parity, p, ghost, static_cast<S*>(buf), c0, cnt);
+  else if (dtype == 1)
+    k_populations<S, double, false, SET><<<grid, kMomThreads, 0, s>>>(P, parity, p, ghost, static_cast<double*>(buf), c0, cnt);
+  else
+    k_populations<S, float, false, SET><<<grid, kMomThreads, 0, s>>>(P, parity, p, ghost, static_cast<float*>(buf), c0, cnt);
 }
 
 // Raw stored values of storage slot `slot` of all fields on plane z, [k][y][x]; T is an
@@ -226,24 +261,16 @@ cudaError_t launch_sensor(const DomainConst& P, int store, int parity, const voi
   return cudaGetLastError();
 }
 
-cudaError_t launch_pop_get(const DomainConst& P, int store, int parity, const void* pop,
-                           const float* ghost, int k, int i, void* out, int dtype, cudaStream_t s) {
-  const int block = 256, grid = grid_for(P.ncell, block);
-  switch (store) {
-    case 0: k_pop_get<float><<<grid, block, 0, s>>>(P, parity, (const float*)pop, ghost, k, i, out, dtype); break;
-    case 1: k_pop_get<__half><<<grid, block, 0, s>>>(P, parity, (const __half*)pop, ghost, k, i, out, dtype); break;
-    default: k_pop_get<__nv_bfloat16><<<grid, block, 0, s>>>(P, parity, (const __nv_bfloat16*)pop, ghost, k, i, out, dtype); break;
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pop_set(const DomainConst& P, int store, int parity, void* pop, int k, int i,
-                           const void* in, int dtype, cudaStream_t s) {
-  const int block = 256, grid = grid_for(P.ncell, block);
-  switch (store) {
-    case 0: k_pop_set<float><<<grid, block, 0, s>>>(P, parity, (float*)pop, k, i, in, dtype); break;
-    case 1: k_pop_set<__half><<<grid, block, 0, s>>>(P, parity, (__half*)pop, k, i, in, dtype); break;
-    default: k_pop_set<__nv_bfloat16><<<grid, block, 0, s>>>(P, parity, (__nv_bfloat16*)pop, k, i, in, dtype); break;
+cudaError_t launch_populations(const DomainConst& P, int store, int parity, void* pop,
+                               const float* ghost, void* buf, int dtype, int set, long long c0,
+                               long long cnt, cudaStream_t s) {
+  switch (store * 2 + set) {
+    case 0: launch_populations_t<float, false>(P, parity, pop, ghost, buf, dtype, c0, cnt, s); break;
+    case 1: launch_populations_t<float, true>(P, parity, pop, ghost, buf, dtype, c0, cnt, s); break;
+    case 2: launch_populations_t<__half, false>(P, parity, pop, ghost, buf, dtype, c0, cnt, s); break;
+    case 3: launch_populations_t<__half, true>(P, parity, pop, ghost, buf, dtype, c0, cnt, s); break;
+    case 4: launch_populations_t<__nv_bfloat16, false>(P, parity, pop, ghost, buf, dtype, c0, cnt, s); break;
+    default: launch_populations_t<__nv_bfloat16, true>(P, parity, pop, ghost, buf, dtype, c0, cnt, s); break;
   }
   return cudaGetLastError();
 }

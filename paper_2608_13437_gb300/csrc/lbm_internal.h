@@ -181,11 +181,12 @@ cudaError_t launch_moments(const DomainConst& P, int store, int parity, const vo
 cudaError_t launch_sensor(const DomainConst& P, int store, int parity, const void* pop,
                           const float* ghost, void* out, int out_f64, long long c0, long long cnt,
                           cudaStream_t s);
-// One population array (k, i) in canonical order, decoded (dtype F32/F64) or native.
-cudaError_t launch_pop_get(const DomainConst& P, int store, int parity, const void* pop,
-                           const float* ghost, int k, int i, void* out, int dtype, cudaStream_t s);
-cudaError_t launch_pop_set(const DomainConst& P, int store, int parity, void* pop, int k, int i,
-                           const void* in, int dtype, cudaStream_t s);
+// All 98 population arrays of cells [c0, c0 + cnt) (c0 a multiple of 32) in canonical
+// order, buf[k][i][cnt], decoded (dtype F32/F64) or native: copied into buf (set = 0) or
+// from buf (set = 1).
+cudaError_t launch_populations(const DomainConst& P, int store, int parity, void* pop,
+                               const float* ghost, void* buf, int dtype, int set, long long c0,
+                               long long cnt, cudaStream_t s);
 // Raw stored values of storage slot `slot` on plane z, all fields, [k][y][x] in the
 // storage's element size: copied into buf (set = 0) or from buf (set = 1).
 cudaError_t launch_plane(const DomainConst& P, int store, void* pop, int z, int slot, void* buf,

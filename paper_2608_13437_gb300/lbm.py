@@ -87,6 +87,7 @@ _SIGNATURES = {
     "lbm_init_riemann": (_IP, [_VP, _IP, _IP, _DP, _DP]),
     "lbm_init_fields": (_IP, [_VP, _VP, _IP, _IP]),
     "lbm_init_state": (_IP, [_VP, _VP, _IP, _IP]),
+    "lbm_init_fields_arrays": (_IP, [_VP, ctypes.POINTER(_VP), _IP]),
     "lbm_step": (_IP, [_VP, _IP]),
     "lbm_synchronize": (_IP, [_VP]),
     "lbm_moments": (_IP, [_VP, _IP, _VP, _IP, _IP]),
@@ -239,6 +240,14 @@ class Domain:
         check(lib().lbm_init_riemann(self._h, axis, i_split, L, R))
 
     def init_fields(self, rho, ux, uy, uz, p, dtype=np.float64):
+        if np.dtype(dtype) in (np.float32, np.float64):
+            # each array goes to the device as it is
+            arrs = [np.ascontiguousarray(np.broadcast_to(a, self.shape), dtype=dtype)
+                    for a in (rho, ux, uy, uz, p)]
+            ptrs = (ctypes.c_void_p * 5)(*[a.ctypes.data for a in arrs])
+            check(lib().lbm_init_fields_arrays(self._h, ptrs,
+                                               DT_F64 if arrs[0].dtype == np.float64 else DT_F32))
+            return
         arr = np.ascontiguousarray(np.stack([np.broadcast_to(a, self.shape) for a in
                                              (rho, ux, uy, uz, p)]), dtype=dtype)
         check(lib().lbm_init_fields(self._h, _np_ptr(arr), 0,
