@@ -365,7 +365,10 @@ lbm_status lbm_set_kernel_config(lbm_handle* h, int block_x, int variant);
  * updating tile t first asks L2, with one bulk prefetch per slot run, for the slot
  * blocks that the warp on tile t + tiles will read, so that warp's loads meet L2
  * instead of DRAM (an implementation choice; the paper has no counterpart). 0 turns
- * it off; the staged and batched forms ignore it. The default is 1024 tiles for 16-bit storage and 0 for FP32; lbm_autotune
+ * it off; the staged and batched forms ignore it. The default is 1024 tiles for 16-bit
+ * storage and 0 for FP32; until this call or lbm_autotune fixes a distance, the steps
+ * follow the size of the state instead of the default: none when the L2 holds the
+ * populations, else 1024 tiles (16-bit) or 256 (FP32). lbm_autotune
  * chooses among 0, 512, 1024 and 2048. Populations are bit-identical with any
  * distance. LBM_E_INVAL for tiles < 0 or > 2^20 or a NULL handle. */
 lbm_status lbm_set_prefetch(lbm_handle* h, int tiles);

@@ -174,6 +174,8 @@ struct lbm_handle {
   bool nonfinite = false;
   int block_x = 64;
   int variant = 0;             // step kernel: register budget (0, 1) or staged form (2-4)
+  int pf_auto = 0;             // L2 prefetch distance while nobody has chosen one (see auto_prefetch)
+  bool pf_chosen = false;      // by lbm_set_prefetch or lbm_autotune: then P.pf_tiles
   int staged_grid = 0;         // persistent grid of the staged forms
   bool stalled = false;        // a step gave up a wait inside its kernel (flag bit 2)
   bool skip_next_copy = false; // test hook: the next direct staged step skips one copy
@@ -223,11 +225,18 @@ int effective_block(const lbm_handle* h) {
   return b > need ? need : b;
 }
 
+// The domain constants a step kernel gets: with the prefetch distance in effect.
+DomainConst step_const(const lbm_handle* h) {
+  DomainConst P = h->P;
+  if (!h->pf_chosen) P.pf_tiles = h->pf_auto;
+  return P;
+}
+
 cudaError_t step_launch(lbm_handle* h, int parity, cudaStream_t s) {
   if (h->variant >= kFirstStagedVariant)
     return launch_step_staged(h->P, h->prm.store, parity, h->pop, h->flag, h->variant,
                               h->staged_grid, 0, s);
-  return launch_step(h->P, h->prm.store, parity, h->pop, h->ghost, h->flag, effective_block(h),
+  return launch_step(step_const(h), h->prm.store, parity, h->pop, h->ghost, h->flag, effective_block(h),
                      h->variant, s);
 }
 
@@ -266,6 +275,22 @@ lbm_status ensure_graphs(lbm_handle* h) {
   if (s != LBM_OK) return s;
   h->graphs_valid = true;
   return LBM_OK;
+}
+
+// L2 prefetch distance by the state's size (measured, block 64, 170 registers). A state that
+// the L2 holds has nothing to fetch, and the hint costs instructions and L2 traffic: 64^3
+// FP16 13.7 us with 1024 tiles, 13.1 without; 80^3 FP16 (100 MB) 35.5 and 34.7. Beyond it
+// 16-bit storage needs one: 96^3 FP16 61.7 us without, 53.9 with 1024 tiles; FP32 gains a
+// little at a short distance: 256^3 1857 us without, 1847 with 256 tiles, 128^3 233.0 and
+// 232.2, 150 x 100 x 60 101.9 and 102.0.
+int auto_prefetch(int store, size_t pop_bytes, int device) {
+  int l2 = 0;
+  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, device) != cudaSuccess) {
+    cudaGetLastError();
+    l2 = 0;
+  }
+  if (pop_bytes <= (size_t)l2 / 100 * 85) return 0;
+  return store == LBM_STORE_F32 ? 256 : kDefaultPrefetch16;
 }
 
 // Sets up the resident form if the domain is small enough for the device. Its memory is a
@@ -434,6 +459,7 @@ lbm_status lbm_create(const lbm_params* p, lbm_handle** out) {
   h->variant = 0;
   h->ncell = h->P.ncell;
   h->pop_bytes = lbm_population_bytes(p);
+  h->pf_auto = auto_prefetch(p->store, h->pop_bytes, device);
   for (int k = 0; k < kF; ++k) h->scale[k] = 1.0;
   h->stream = static_cast<cudaStream_t>(p->cuda_stream);
   auto cleanup = [&](lbm_status st) {
@@ -914,7 +940,7 @@ lbm_status lbm_step_diag(lbm_handle* h, int n, lbm_diag_t* out) {
   }
   if (!h->ev_diag) LBM_CUDA(cudaEventCreateWithFlags(&h->ev_diag, cudaEventDisableTiming));
   const long long step0 = h->step;
-  LBM_CUDA(launch_step_diag(h->P, h->prm.store, (int)(h->step & 1), h->pop, h->ghost, h->flag,
+  LBM_CUDA(launch_step_diag(step_const(h), h->prm.store, (int)(h->step & 1), h->pop, h->ghost, h->flag,
                             h->ufield, h->wrec, bx, h->stream));
   h->step += 1;
   LBM_CUDA(launch_diag_records(h->P, h->wrec, nrec, h->ufield, h->partials, h->dout, h->stream));
@@ -1046,6 +1072,7 @@ lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out) {
   float best = 1e30f;
   int best_b = h->block_x, best_v = h->variant, best_grid = h->staged_grid, tried = 0;
   int best_pf = h->P.pf_tiles;
+  h->pf_chosen = true;
   cudaError_t err = cudaSuccess;
   for (const Cand& c : cands) {
     int grid = 0;
@@ -1157,6 +1184,7 @@ lbm_status lbm_set_prefetch(lbm_handle* h, int tiles) {
   if (tiles < 0 || tiles > kMaxPrefetch)
     return fail(LBM_E_INVAL, "prefetch distance must be 0 to %d tiles", kMaxPrefetch);
   h->P.pf_tiles = tiles;
+  h->pf_chosen = true;
   h->graphs_valid = false;
   return LBM_OK;
 }
