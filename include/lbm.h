@@ -468,7 +468,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int steps_per_trial, int* tile_cells
 /* L2 prefetch distance of the persistent kernel, in tiles (an implementation choice;
  * the paper has no counterpart): a warp starting an item asks L2 for the slot blocks
  * of the item that many tiles ahead in the claim order, in the pattern of
- * lbm_set_prefetch. 0 turns it off; the default is 1024 for 16-bit storage and 0 for
+ * lbm_set_prefetch. 0 turns it off; the default is 1024 for 16-bit storage (not used on
+ * a pool that the L2 holds, until this call or the autotuner fixes a distance) and 0 for
  * FP32. Populations are bit-identical with any distance. LBM_E_INVAL for tiles < 0 or
  * > 2^20 or a NULL batch. */
 lbm_status lbm_batch_set_prefetch(lbm_batch* b, int tiles);
