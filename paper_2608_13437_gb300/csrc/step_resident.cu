@@ -20,9 +20,9 @@
 //     odd tags. A neighbour overwrites an inbox two steps later; by then it has received
 //     this brick's packets of the step between, which were sent after the inbox was read.
 //   * The same dependence orders memory at both ends of the launch: a brick stores its
-//     populations only after it has received a step's packets from its neighbours, which
-//     they send after they have loaded theirs, and a location is loaded and stored by one
-//     brick and its direct neighbours along that population's axis alone.
+//     populations after the last step, when it has received packets from its neighbours,
+//     which they send after they have loaded theirs, and a location is loaded and stored by
+//     one brick and its direct neighbours along that population's axis alone.
 //   * Launched cooperatively (every block resident, or the launch fails). A poll gives up
 //     after a bounded number of tries; the block then sets flag bit 2 and returns without
 //     storing, its neighbours run out the same way, and the host reports LBM_E_TIMEOUT.
@@ -152,8 +152,19 @@ __device__ __forceinline__ uint4 packet_load(const uint4* p) {
 // microsecond), so about a second.
 constexpr int kMaxPolls = 1 << 21;
 
-template <typename S, bool SR>
-__global__ void __launch_bounds__(kResidentMaxThreads, 1)
+// Exchange buffers of a block: two where 200 KB of shared memory hold them, which saves a
+// barrier per step.
+template <typename S, int MAXT>
+constexpr int exchange_buffers() {
+  return (size_t)MAXT * 13 * kF * sizeof(S) <= 200 * 1024 ? 2 : 1;
+}
+
+// MAXT: threads of the largest block. 256 leave 255 registers a thread, which lets one warp
+// per scheduler overlap more of its own latencies: 1024 x 4 x 4 FP32 2.13 -> 1.78 us a step,
+// 256 x 4 x 3 1.94 -> 1.74, 32^3 3.21 -> 3.10; 384 leave 168. (The second exchange buffer
+// and the last step's stores outside the loop: 1.68, 1.59 and 2.98.)
+template <typename S, bool SR, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1)
     k_resident(const DomainConst P, const ResidentPlan R, S* __restrict__ pop,
                const float* __restrict__ ghost, unsigned* __restrict__ flag,
                uint4* __restrict__ inbox, unsigned* __restrict__ epochs, int parity0, int steps) {
@@ -162,9 +173,12 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 1)
   constexpr int NW = Words<S>::n, NP = Words<S>::packets;
   extern __shared__ __align__(16) unsigned char smem[];
   const int T = blockDim.x, tid = threadIdx.x;
-  V4* const s4 = reinterpret_cast<V4*>(smem);              // [6][3][T]
-  V2* const s2 = reinterpret_cast<V2*>(s4 + 6 * 3 * T);    // [6][T]
-  uint2* const table = reinterpret_cast<uint2*>(s2 + 6 * T);  // [packet sets of the brick]
+  // exchange buffers (one, or two for even and odd tags), the rest populations of the last
+  // step, and the table of the packet sets that arrive from outside
+  constexpr int kBuffers = exchange_buffers<S, MAXT>();
+  V4* const x4 = reinterpret_cast<V4*>(smem);                  // [kBuffers][6][3][T], rest [3][T]
+  V2* const x2 = reinterpret_cast<V2*>(x4 + (6 * kBuffers + 1) * 3 * T);  // [kBuffers][6][T], [T]
+  uint2* const table = reinterpret_cast<uint2*>(x2 + (6 * kBuffers + 1) * T);
   // brick and cell
   const int bx = blockIdx.x % R.g[0], by = blockIdx.x / R.g[0] % R.g[1],
             bz = blockIdx.x / (R.g[0] * R.g[1]);
@@ -231,21 +245,28 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 1)
   bool bad = false;
   // Where the state is stored after the last step: the read position of the new parity.
   const int parity1 = (parity0 + steps) & 1;
-  auto store_words = [&](int i, const unsigned (&w)[NW]) {
+  auto store_groups = [&](int i, const V4* v4, const V2* v2) {
     const long long cell = src_cell(P, c, parity1, i);
     if (!LBM_CHECK(P, cell >= 0 && cell < P.ntile * kTile)) return;
     S* base = pop + tile_start(cell);
     const int lane = (int)(cell & (kTile - 1));
     const int sl = parity1 ? opp(i) : i;
 #pragma unroll
-    for (int g = 0; g < 3; ++g) *reinterpret_cast<V4*>(base + group_offset(sl, g, lane)) = words4<S>(w, g);
-    *reinterpret_cast<V2*>(base + group_offset(sl, 3, lane)) = words2<S>(w);
+    for (int g = 0; g < 3; ++g) *reinterpret_cast<V4*>(base + group_offset(sl, g, lane)) = v4[g * T + tid];
+    *reinterpret_cast<V2*>(base + group_offset(sl, 3, lane)) = v2[tid];
   };
+  V4* const rest4 = x4 + 6 * kBuffers * 3 * T;
+  V2* const rest2 = x2 + 6 * kBuffers * T;
+  V4* s4 = x4;
+  V2* s2 = x2;
 
 #pragma unroll 1
   for (int t = 0; t < steps; ++t) {
     const unsigned tag = epoch + (unsigned)t + 1u;
-    const bool last = t + 1 == steps;
+    if (kBuffers == 2) {
+      s4 = x4 + (tag & 1u) * (6 * 3 * T);
+      s2 = x2 + (tag & 1u) * (6 * T);
+    }
     if (active) {
       if (P.bc_x) {  // held x ends: the inward populations come from the ghost layer
         if (x == 0) {
@@ -266,8 +287,12 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 1)
         unsigned w[NW];
         pack_dir<S, SR>(P, d, i, &dz, w);
         if (i == 0) {
-          if (last) store_words(0, w);
-          else if constexpr (!std::is_same<S, float>::value) unpack_dir<S>(P, w, d, 0);
+          if (t + 1 == steps) {
+#pragma unroll
+            for (int g = 0; g < 3; ++g) rest4[g * T + tid] = words4<S>(w, g);
+            rest2[tid] = words2<S>(w);
+          }
+          if constexpr (!std::is_same<S, float>::value) unpack_dir<S>(P, w, d, 0);
           continue;
         }
         const int dst = to[i - 1];
@@ -324,7 +349,10 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 1)
       for (int g = 0; g < 3; ++g) s4[(in.y >> 16) * 3 * T + g * T + (in.y & 0xFFFFu)] = words4<S>(w, g);
       s2[(in.y >> 16) * T + (in.y & 0xFFFFu)] = words2<S>(w);
     }
-    __syncthreads();
+    if (__syncthreads_or(dead)) {  // a block whose wait ran out stops here
+      if (tid == 0) atomicOr(flag, 2u);
+      return;
+    }
     if (active) {
 #pragma unroll
       for (int i = 1; i < kQ; ++i) {
@@ -333,34 +361,38 @@ __global__ void __launch_bounds__(kResidentMaxThreads, 1)
         for (int g = 0; g < 3; ++g) a[g] = s4[((i - 1) * 3 + g) * T + tid];
         unsigned w[NW];
         from_groups<S>(a, s2[(i - 1) * T + tid], w);
-        if (last) store_words(i, w);
-        else unpack_dir<S>(P, w, d, i);
+        unpack_dir<S>(P, w, d, i);
       }
     }
-    // everyone is done with the exchange buffer; a block whose wait ran out stops here
-    if (__syncthreads_or(dead)) {
-      if (tid == 0) atomicOr(flag, 2u);
-      return;
-    }
+    // One buffer: everyone is done with it before the next step writes it. With two, the
+    // next step's barrier separates this step's reads from the writes two steps on.
+    if (kBuffers == 1) __syncthreads();
+  }
+  // the state as the last exchange left it, words as they are
+  if (active) {
+    store_groups(0, rest4, rest2);
+#pragma unroll
+    for (int i = 1; i < kQ; ++i) store_groups(i, s4 + (i - 1) * 3 * T, s2 + (i - 1) * T);
   }
   if (bad) atomicOr(flag, 1u);
   if (tid == 0) epochs[blockIdx.x] = epoch + (unsigned)steps;
 }
 
-// Shared memory of a block: six directions of every cell, and the table (at most six
-// packet sets a cell).
-template <typename S>
+// Shared memory of a block: the exchange buffers, the rest populations, and the table (at
+// most six packet sets a cell).
+template <typename S, int MAXT>
 constexpr size_t smem_bytes(int threads) {
-  return (size_t)threads * 6 * (kF * sizeof(S) + sizeof(uint2));
+  return (size_t)threads * ((6 * exchange_buffers<S, MAXT>() + 1) * kF * sizeof(S) + 6 * sizeof(uint2));
 }
 
-template <typename S, bool SR>
-cudaError_t launch_t(const DomainConst& P, const ResidentPlan& R, void* pop, const float* ghost,
+template <typename S, bool SR, int MAXT>
+cudaError_t launch_threads(const DomainConst& P, const ResidentPlan& R, void* pop, const float* ghost,
                      unsigned* flag, void* inbox, unsigned* epochs, int parity, int steps,
                      cudaStream_t s) {
-  const size_t smem = smem_bytes<S>(R.threads);
-  cudaError_t e = cudaFuncSetAttribute(k_resident<S, SR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem_bytes<S>(kResidentMaxThreads));
+  const size_t smem = smem_bytes<S, MAXT>(R.threads);
+  cudaError_t e = cudaFuncSetAttribute(k_resident<S, SR, MAXT>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem_bytes<S, MAXT>(MAXT));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(R.blocks());
@@ -372,8 +404,17 @@ cudaError_t launch_t(const DomainConst& P, const ResidentPlan& R, void* pop, con
   attr.val.cooperative = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_resident<S, SR>, P, R, static_cast<S*>(pop), ghost, flag,
+  return cudaLaunchKernelEx(&cfg, k_resident<S, SR, MAXT>, P, R, static_cast<S*>(pop), ghost, flag,
                             static_cast<uint4*>(inbox), epochs, parity, steps);
+}
+
+template <typename S, bool SR>
+cudaError_t launch_t(const DomainConst& P, const ResidentPlan& R, void* pop, const float* ghost,
+                     unsigned* flag, void* inbox, unsigned* epochs, int parity, int steps,
+                     cudaStream_t s) {
+  if (R.threads <= 256)
+    return launch_threads<S, SR, 256>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
+  return launch_threads<S, SR, kResidentMaxThreads>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
 }
 
 }  // namespace
@@ -382,25 +423,28 @@ bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R) {
   if (!P.collide || P.ncell > (long long)sms * kResidentMaxThreads) return false;
   const int n[3] = {P.nx, P.ny, P.nz};
   long long best = -1;
-  for (int bx = 1; bx <= std::min(n[0], kResidentMaxThreads); ++bx) {
-    const int gx = (n[0] + bx - 1) / bx;
-    if (gx > sms) continue;
-    for (int by = 1; by <= std::min(n[1], kResidentMaxThreads / bx); ++by) {
-      const int gy = (n[1] + by - 1) / by;
-      if (gx * gy > sms) continue;
-      for (int bz = 1; bz <= std::min(n[2], kResidentMaxThreads / (bx * by)); ++bz) {
-        const int gz = (n[2] + bz - 1) / bz;
-        if (gx * gy * gz > sms) continue;
+  // every number of bricks along an axis that its side can be cut into evenly (the smallest
+  // brick for that number)
+  auto side = [](int n, int g) { return (n + g - 1) / g; };
+  for (int gx = 1; gx <= std::min(n[0], sms); ++gx) {
+    const int bx = side(n[0], gx);
+    if (side(n[0], bx) != gx || bx > kResidentMaxThreads) continue;
+    for (int gy = 1; gy <= std::min(n[1], sms / gx); ++gy) {
+      const int by = side(n[1], gy);
+      if (side(n[1], by) != gy || bx * by > kResidentMaxThreads) continue;
+      for (int gz = 1; gz <= std::min(n[2], sms / (gx * gy)); ++gz) {
+        const int bz = side(n[2], gz);
+        if (side(n[2], bz) != gz || bx * by * bz > kResidentMaxThreads) continue;
         const int face[3] = {gx > 1 ? by * bz : 0, gy > 1 ? bx * bz : 0, gz > 1 ? bx * by : 0};
-        // Nanoseconds of a step, fitted to a sweep of 80 bricks of nine domains (FP32, within
-        // about 10 %): one warp's latency, the issue of the brick's warps, a trip to the
-        // neighbours along each axis that leaves the brick, and one more poll for every
-        // further packet set a thread fetches.
+        // Nanoseconds of a step, fitted to sweeps of 80 bricks of nine domains (FP32, within
+        // about 15 %): one warp's latency (more with 168 registers), the issue of the brick's
+        // warps, a trip to the neighbours along each axis that leaves the brick, the packets,
+        // and one more poll for every further set of them that a thread fetches.
         const long long warps = (bx * by * bz + 31) / 32;
         const long long sets = 2LL * (face[0] + face[1] + face[2]), threads = 32 * warps;
-        long long cost = 1200 + 150 * warps;
+        long long cost = (warps <= 8 ? 900 : 1300) + 150 * warps;
         for (int a = 0; a < 3; ++a) cost += face[a] ? 300 : 0;
-        if (sets > 0) cost += 400 * ((sets + threads - 1) / threads - 1);
+        if (sets > 0) cost += 300 * ((sets + threads - 1) / threads - 1) + 100 * sets / threads;
         if (best < 0 || cost < best) {
           best = cost;
           *R = ResidentPlan{{bx, by, bz}, {gx, gy, gz}, (int)(32 * warps),
@@ -409,12 +453,12 @@ bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R) {
       }
     }
   }
-  // Against the plain kernel's nanoseconds at these sizes, fitted to the same domains: 2.2 us
-  // at 4 thousand cells, 3.8 at 33 thousand (FP32); 16-bit storage 2.4-2.6 and 3.0-3.1 us,
-  // and its resident form is 0.1 to 0.4 us below the model. Resident, FP32: 2.06 us at
-  // 1024 x 4 x 4 (plain 3.08), 3.21 at 32^3 (3.78), 4.47 at 38^3 (6.17), 2.48 at 16^3 (2.18).
+  // Against the plain kernel's nanoseconds at these sizes, fitted to the same domains (FP32);
+  // with 16-bit storage the plain kernel was slower on all of them. Resident against plain,
+  // FP32: 1.6 us at 1024 x 4 x 4 (3.1), 2.95 at 32^3 (3.8), 4.1 at 38^3 (5.5), 1.95 at 16^3
+  // (2.2), 2.05 at 20 x 12 x 9 (2.2); FP16 1.6 (2.8), 2.6 (3.1), 3.8 (4.6), 2.0 (2.6).
   if (best < 0) return false;
-  return store == 0 ? best + 150 < 2050 + 52 * P.ncell / 1000 : best - 200 < 2300 + 25 * P.ncell / 1000;
+  return store != 0 || best < 2050 + 52 * P.ncell / 1000;
 }
 
 size_t resident_inbox_bytes(const ResidentPlan& R, int store) {
