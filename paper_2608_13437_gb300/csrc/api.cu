@@ -84,6 +84,8 @@ void fill_const(const lbm_params* p, double dt, double tau_R, double tau_q, Doma
   P->bc_x = p->bc_x;
   P->ncell = (long long)p->nx * p->ny * p->nz;
   P->ntile = tile_count(P->ncell);
+  P->by_nx = fast_div((unsigned)p->nx);
+  P->by_ny = fast_div((unsigned)p->ny);
   const double c = p->dx / dt;
   P->c = (float)c;
   P->inv_c = (float)(1.0 / c);

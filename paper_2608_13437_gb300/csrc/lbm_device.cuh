@@ -29,6 +29,24 @@ constexpr float kSutherlandT = 0.4042f;
 
 __host__ __device__ constexpr int opp(int i) { return i == 0 ? 0 : ((i & 1) ? i + 1 : i - 1); }
 
+// Division of n < 2^31 by a constant d >= 1 as one wide multiplication and a shift:
+// n / d = (n m) >> s with l = ceil(log2 d), s = 31 + l, m = floor(2^s / d) + 1 < 2^32. The
+// excess of m over 2^s / d is at most 1 <= 2^l / d, so n m / 2^s exceeds n / d by less than
+// 1 / d and its floor is exact (Granlund and Montgomery 1994). The compiler's own 32-bit
+// division is a chain of about 20 instructions in front of every load.
+struct FastDiv {
+  unsigned m;
+  int s;
+};
+inline FastDiv fast_div(unsigned d) {
+  int l = 0;
+  while ((1ull << l) < d) ++l;
+  return FastDiv{(unsigned)((1ull << (31 + l)) / d + 1), 31 + l};
+}
+__device__ __forceinline__ unsigned div_by(unsigned n, const FastDiv& f) {
+  return (unsigned)(((unsigned long long)n * f.m) >> f.s);
+}
+
 // Constants of one domain, passed by value to every kernel.
 struct DomainConst {
   int nx, ny, nz, bc_x;
@@ -50,6 +68,7 @@ struct DomainConst {
   int sround;         // 16-bit storage rounds stochastically (1) or to nearest (0)
   int pf_tiles;       // L2 prefetch distance of the plain step kernel (0: off)
   int eso;            // storage map: 0 AA pattern, 1 esoteric twist (slots 2, 4, 6 shifted)
+  FastDiv by_nx, by_ny;  // division of cell indices by nx and of row indices by ny
   double dx64;        // dx in FP64 (the diagnostics' gradient pass takes 1/dx from it)
   unsigned* check;    // checked builds: count of population addresses found outside the buffer
 };

@@ -9,14 +9,13 @@
 
 namespace lbm {
 
-// (x, y, z) of a linear cell index; cell counts are below 2^31, so 32-bit unsigned
-// division suffices (much cheaper than 64-bit).
+// (x, y, z) of a linear cell index (cell counts are below 2^31).
 __device__ __forceinline__ void cell_xyz(const DomainConst& P, long long cell, int& x, int& y,
                                          int& z) {
   const unsigned c = (unsigned)cell;
-  const unsigned yz = c / (unsigned)P.nx;
+  const unsigned yz = div_by(c, P.by_nx);
   x = (int)(c - yz * (unsigned)P.nx);
-  const unsigned zz = yz / (unsigned)P.ny;
+  const unsigned zz = div_by(yz, P.by_ny);
   y = (int)(yz - zz * (unsigned)P.ny);
   z = (int)zz;
 }
@@ -33,12 +32,12 @@ __device__ __forceinline__ void tile_xyz(const DomainConst& P, long long t, int 
       ++y;
     }
   } else {
-    const int rows = x / P.nx;
+    const int rows = (int)div_by((unsigned)x, P.by_nx);
     x -= rows * P.nx;
     y += rows;
   }
   if (y >= P.ny) {  // rows shorter than a tile may end several planes
-    const int planes = y / P.ny;
+    const int planes = (int)div_by((unsigned)y, P.by_ny);
     y -= planes * P.ny;
     z += planes;
   }
