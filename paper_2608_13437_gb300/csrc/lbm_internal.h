@@ -111,7 +111,8 @@ constexpr int kResidentMaxThreads = 384;  // cells of a brick at most: 170 regis
 struct ResidentPlan {
   int b[3], g[3];
   int threads;  // of a block: the brick's cells rounded up to whole warps
-  int face;     // cells of the largest face through which bricks exchange
+  int sets;     // cells of the faces through which a brick receives, both directions of an axis
+  int first[3]; // the first of them of each axis
   int blocks() const { return g[0] * g[1] * g[2]; }
 };
 // Chooses the bricks for `sms` blocks resident at once; false if the domain does not fit or

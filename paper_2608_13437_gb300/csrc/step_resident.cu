@@ -200,8 +200,13 @@ __global__ void __launch_bounds__(MAXT, 1)
     to[2 * a] = l + 1 < width ? tid + stride : (whole ? tid - (width - 1) * stride : kOut);
     to[2 * a + 1] = l > 0 ? tid - stride : (whole ? tid + (width - 1) * stride : kOut);
   }
-  // offset of packet 0 of direction i to the face cell f of brick b's inbox 0
-  auto slot = [&](int b, int i, int f) { return (unsigned)((b * 12 + (i - 1)) * NP * R.face + f); };
+  // offset of packet 0 of direction i to the face cell f of brick b's inbox 0: an inbox
+  // holds [packet][set], the sets of the axes that leave the brick one after the other
+  auto slot = [&](int b, int i, int f) {
+    const int a = (i - 1) >> 1;
+    const int face = a == 0 ? R.b[1] * R.b[2] : (a == 1 ? R.b[0] * R.b[2] : R.b[0] * R.b[1]);
+    return (unsigned)(b * 2 * NP * R.sets + R.first[a] + ((i - 1) & 1) * face + f);
+  };
   auto neighbour = [&](int i) {  // the brick that direction i leads to
     const int a = (i - 1) >> 1, s = (i & 1) ? 1 : -1;
     const int c = a == 0 ? bx : (a == 1 ? by : bz);
@@ -299,10 +304,10 @@ __global__ void __launch_bounds__(MAXT, 1)
         if (dst == kOut) {
           // the destination cell has the same place on its brick's face
           const int f = i < 3 ? ly + R.b[1] * lz : (i < 5 ? lx + R.b[0] * lz : lx + R.b[0] * ly);
-          uint4* p = inbox + slot(neighbour(i), i, f) + (tag & 1u) * (6u * NP * R.face);
+          uint4* p = inbox + slot(neighbour(i), i, f) + (tag & 1u) * (unsigned)(NP * R.sets);
 #pragma unroll
           for (int q = 0; q < NP; ++q)
-            packet_store(p + (size_t)q * R.face, w[3 * q], 3 * q + 1 < NW ? w[3 * q + 1] : tag,
+            packet_store(p + (size_t)q * R.sets, w[3 * q], 3 * q + 1 < NW ? w[3 * q + 1] : tag,
                          3 * q + 2 < NW ? w[3 * q + 2] : tag, tag);
         } else {
 #pragma unroll
@@ -318,12 +323,12 @@ __global__ void __launch_bounds__(MAXT, 1)
     bool dead = false;
     for (int e = tid; e < n_in; e += T) {
       const uint2 in = table[e];
-      const uint4* p = inbox + in.x + (tag & 1u) * (6u * NP * R.face);
+      const uint4* p = inbox + in.x + (tag & 1u) * (unsigned)(NP * R.sets);
       unsigned w[3 * NP];
       for (int tries = 0;; ++tries) {
         uint4 m[NP];
 #pragma unroll
-        for (int q = 0; q < NP; ++q) m[q] = packet_load(p + (size_t)q * R.face);
+        for (int q = 0; q < NP; ++q) m[q] = packet_load(p + (size_t)q * R.sets);
         bool ok = true;
 #pragma unroll
         for (int q = 0; q < NP; ++q) {
@@ -447,8 +452,8 @@ bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R) {
         if (sets > 0) cost += 300 * ((sets + threads - 1) / threads - 1) + 100 * sets / threads;
         if (best < 0 || cost < best) {
           best = cost;
-          *R = ResidentPlan{{bx, by, bz}, {gx, gy, gz}, (int)(32 * warps),
-                            std::max(1, std::max(face[0], std::max(face[1], face[2])))};
+          *R = ResidentPlan{{bx, by, bz}, {gx, gy, gz}, (int)threads, (int)std::max(1LL, sets),
+                            {0, 2 * face[0], 2 * (face[0] + face[1])}};
         }
       }
     }
@@ -463,7 +468,7 @@ bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R) {
 
 size_t resident_inbox_bytes(const ResidentPlan& R, int store) {
   const int packets = store == 0 ? Words<float>::packets : Words<__half>::packets;
-  return (size_t)R.blocks() * 2 * 6 * packets * R.face * sizeof(uint4);
+  return (size_t)R.blocks() * 2 * packets * R.sets * sizeof(uint4);
 }
 
 cudaError_t launch_resident(const DomainConst& P, const ResidentPlan& R, int store, int parity,
