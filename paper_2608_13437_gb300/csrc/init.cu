@@ -18,6 +18,7 @@
 // The fluxes of the equilibrium are not deviations; they are evaluated in FP32 from the
 // cell's primitives. Populations are written with the step kernels' vector stores (one
 // warp fills one 32-cell tile).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 
@@ -179,32 +180,41 @@ __device__ void initial_cell(const DomainConst& P, const InitSpec& sp, int x, in
   s.heat = mul(P.heat0, r);
 }
 
-// Deviations of the linear equilibrium: d_0 = D/4, d_{+-a} = D/8 +- Phi_a / (2c).
-__device__ __forceinline__ void equilibrium_dev(const DomainConst& P, const InitCell& c,
-                                                float (&dev)[kF][kQ]) {
+// The linear equilibrium's deviations d_0 = D/4, d_{+-a} = D/8 +- Phi_a / (2c), by what
+// they are made of: 56 values a cell are held instead of 98.
+struct Equilibrium {
+  float D[kF], flux[3][kF];  // Phi_a / (2c)
+};
+__device__ __forceinline__ void equilibrium_of(const DomainConst& P, const InitCell& c, Equilibrium& q) {
 #pragma unroll
   for (int k = 0; k < kF; ++k) {
     float fx, fy, fz;
     field_flux<float>(k, c.s, fx, fy, fz);
-    const float e0 = mul(0.25f, c.D[k]), e1 = mul(0.125f, c.D[k]);
-    const float ax = mul(P.half_inv_c, fx), ay = mul(P.half_inv_c, fy), az = mul(P.half_inv_c, fz);
-    dev[k][0] = e0;
-    dev[k][1] = add(e1, ax);
-    dev[k][2] = sub(e1, ax);
-    dev[k][3] = add(e1, ay);
-    dev[k][4] = sub(e1, ay);
-    dev[k][5] = add(e1, az);
-    dev[k][6] = sub(e1, az);
+    q.D[k] = c.D[k];
+    q.flux[0][k] = mul(P.half_inv_c, fx);
+    q.flux[1][k] = mul(P.half_inv_c, fy);
+    q.flux[2][k] = mul(P.half_inv_c, fz);
   }
+}
+__device__ __forceinline__ float equilibrium_dev(const Equilibrium& q, int k, int i) {
+  if (i == 0) return mul(0.25f, q.D[k]);
+  const float e1 = mul(0.125f, q.D[k]), a = q.flux[(i - 1) >> 1][k];
+  return (i & 1) ? add(e1, a) : sub(e1, a);
 }
 
 // mode 0: per-field max |d| into maxbits (for the FP16 scales); mode 1: write the
 // populations (canonical slots: slot i of a cell holds f_i, under the esoteric twist
 // with slots 2, 4, 6 one cell further along +x, +y, +z) and the held-x ghosts, and
 // set *bad (if given) when a cell's state is not finite. Blocks of whole warps, so a
-// warp covers one 32-cell tile.
+// warp covers one 32-cell tile. A direction's 14 values are formed as they are stored, so
+// four blocks fit an SM (three with all 98 values at once; five spill), and the maxima go
+// to memory only where they exceed what is there: one atomic per warp and field, all on 14
+// words, was half of a small domain's time. From five fields, both passes where there are
+// two: 64^3 FP16 240 -> 125 us, 128^3 FP16 520 -> 335, 128^3 FP32 twist 370 -> 280, 512^3
+// FP32 11.9 -> 9.6 ms, which is 52.6 GB written and 2.7 read.
+constexpr int kInitBlocks = 4;
 template <typename S>
-__global__ void __launch_bounds__(128) k_init(const DomainConst P, const InitSpec sp, int mode,
+__global__ void __launch_bounds__(128, kInitBlocks) k_init(const DomainConst P, const InitSpec sp, int mode,
                                               S* __restrict__ pop, float* __restrict__ ghost,
                                               unsigned* __restrict__ maxbits,
                                               unsigned* __restrict__ bad) {
@@ -223,42 +233,42 @@ __global__ void __launch_bounds__(128) k_init(const DomainConst P, const InitSpe
     cell_xyz(P, cell, x, y, z);
     InitCell c;
     initial_cell(P, sp, x, y, z, cell, c);
-    float dev[kF][kQ];
-    equilibrium_dev(P, c, dev);
+    Equilibrium q;
+    equilibrium_of(P, c, q);
     if (mode == 0) {
 #pragma unroll
       for (int k = 0; k < kF; ++k)
 #pragma unroll
-        for (int i = 0; i < kQ; ++i) mx[k] = fmaxf(mx[k], fabsf(dev[k][i]));
+        for (int i = 0; i < kQ; ++i) mx[k] = fmaxf(mx[k], fabsf(equilibrium_dev(q, k, i)));
       continue;
     }
     if (bad) {  // a non-finite input or state ends up in the moments or the fluxes
       float probe = 0.0f;
 #pragma unroll
-      for (int k = 0; k < kF; ++k) probe += dev[k][1] + dev[k][2];
+      for (int k = 0; k < kF; ++k) probe += equilibrium_dev(q, k, 1) + equilibrium_dev(q, k, 2);
       if (!isfinite(probe)) atomicOr(bad, 1u);
     }
     if (!LBM_CHECK(P, cell < P.ntile * kTile)) continue;
-    if (P.eso) {  // esoteric twist: slots 2, 4, 6 live with the cell one step along +x, +y, +z
-      const CellIndex ci = make_index(P, x, y, z);
+    // esoteric twist: slots 2, 4, 6 live with the cell one step along +x, +y, +z
+    CellIndex ci{};
+    if (P.eso) ci = make_index(P, x, y, z);
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) {
-        const long long tc = eso_shifted(i) ? ci.nb[i - 1] : cell;
-        if (!LBM_CHECK(P, tc >= 0 && tc < P.ntile * kTile)) continue;
-        store_dir<S>(P, pop + tile_start(tc), i, (int)(tc & (kTile - 1)), dev, i, nullptr);
-      }
-    } else {
-      S* base = pop + tile_start(cell);
-      const int lane = (int)(cell & (kTile - 1));
+    for (int i = 0; i < kQ; ++i) {
+      const long long tc = P.eso && eso_shifted(i) ? ci.nb[i - 1] : cell;
+      if (!LBM_CHECK(P, tc >= 0 && tc < P.ntile * kTile)) continue;
+      float v[kF];
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) store_dir<S>(P, base, i, lane, dev, i, nullptr);
+      for (int k = 0; k < kF; ++k) v[k] = equilibrium_dev(q, k, i);
+      store_fields<S>(P, pop + tile_start(tc), i, (int)(tc & (kTile - 1)), v, nullptr);
     }
     if (P.bc_x && ghost) {
       const long long plane = (long long)y + (long long)P.ny * z;
       if (x == 0)
-        for (int k = 0; k < kF; ++k) ghost[(0 * kF + k) * planes + plane] = dev[k][1];
+#pragma unroll
+        for (int k = 0; k < kF; ++k) ghost[(0 * kF + k) * planes + plane] = equilibrium_dev(q, k, 1);
       if (x == P.nx - 1)
-        for (int k = 0; k < kF; ++k) ghost[(1LL * kF + k) * planes + plane] = dev[k][2];
+#pragma unroll
+        for (int k = 0; k < kF; ++k) ghost[(1LL * kF + k) * planes + plane] = equilibrium_dev(q, k, 2);
     }
   }
   if (mode == 0) {
@@ -266,8 +276,9 @@ __global__ void __launch_bounds__(128) k_init(const DomainConst P, const InitSpe
     for (int k = 0; k < kF; ++k) {
       float m = mx[k];
       for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      // order of non-negative floats = order of their bits
-      if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(&maxbits[k], __float_as_uint(m));
+      // order of non-negative floats = order of their bits; the word only ever grows
+      if ((threadIdx.x & 31) == 0 && m > 0.0f && __float_as_uint(m) > __ldcg(&maxbits[k]))
+        atomicMax(&maxbits[k], __float_as_uint(m));
     }
   }
 }
@@ -339,10 +350,16 @@ __global__ void __launch_bounds__(kMeanThreads) k_field_sums_final(const double*
   if (threadIdx.x < 2) sums[threadIdx.x] = sh[threadIdx.x][0];
 }
 
-int grid_for(long long n, int block) {
-  long long g = (n + block - 1) / block;
-  if (g > 152LL * 32) g = 152LL * 32;
-  return (int)(g < 1 ? 1 : g);
+// Blocks of k_init. The maxima: the resident blocks, so that each warp reduces once (64^3:
+// 100 -> 82 us for both passes of a TGV with 32 blocks per SM before). Populations from a
+// closed form: a block per 128 cells, which the hardware starts in order, so the writes
+// stay close together (512^3 esoteric twist: 8.81 -> 6.94 ms). Populations from fields: 32
+// blocks per SM that stride over the cells; the reads of the next cells start while the
+// last writes drain (512^3: 10.65 -> 9.63 ms).
+int init_grid(long long n, int block, int mode, int kind) {
+  const long long full = (n + block - 1) / block;
+  const long long most = mode == 0 ? 152LL * kInitBlocks : (kind < 2 ? (1LL << 30) : 152LL * 32);
+  return (int)std::max<long long>(1, std::min(full, most));
 }
 
 // 1/(gamma - 1) as a float-float pair.
@@ -417,7 +434,7 @@ void fields_spec(double gamma, int kind, const void* fields, int f64, InitSpec* 
 cudaError_t launch_init(const DomainConst& P, int store, const InitSpec& spec, int mode, void* pop,
                         float* ghost, unsigned* maxbits, unsigned* bad, cudaStream_t s) {
   const int block = 128;
-  const int grid = grid_for(P.ncell, block);
+  const int grid = init_grid(P.ncell, block, mode, spec.kind);
   switch (store) {
     case 0: k_init<float><<<grid, block, 0, s>>>(P, spec, mode, static_cast<float*>(pop), ghost, maxbits, bad); break;
     case 1: k_init<__half><<<grid, block, 0, s>>>(P, spec, mode, static_cast<__half*>(pop), ghost, maxbits, bad); break;

@@ -454,13 +454,10 @@ struct Dither {
 // One direction's 14 fields into the 4 + 4 + 4 + 2 groups of slot `slot`, lane `lane`
 // of the tile at `base`, rounded to nearest or (dz != nullptr) stochastically.
 template <typename S>
-__device__ __forceinline__ void store_dir(const DomainConst& P, S* base, int slot, int lane,
-                                          const float (&d)[kF][kQ], int i, Dither* dz) {
+__device__ __forceinline__ void store_fields(const DomainConst& P, S* base, int slot, int lane,
+                                             const float (&v)[kF], Dither* dz) {
   using V4 = typename Codec<S>::V4;
   using V2 = typename Codec<S>::V2;
-  float v[kF];
-#pragma unroll
-  for (int k = 0; k < kF; ++k) v[k] = d[k][i];
   if constexpr (!std::is_same<S, float>::value) {
     if (dz) {
 #pragma unroll
@@ -478,6 +475,15 @@ __device__ __forceinline__ void store_dir(const DomainConst& P, S* base, int slo
   for (int g = 0; g < 3; ++g)
     *reinterpret_cast<V4*>(base + group_offset(slot, g, lane)) = Codec<S>::enc4(v + 4 * g, P.inv_scale + 4 * g);
   *reinterpret_cast<V2*>(base + group_offset(slot, 3, lane)) = Codec<S>::enc2(v + 12, P.inv_scale + 12);
+}
+
+template <typename S>
+__device__ __forceinline__ void store_dir(const DomainConst& P, S* base, int slot, int lane,
+                                          const float (&d)[kF][kQ], int i, Dither* dz) {
+  float v[kF];
+#pragma unroll
+  for (int k = 0; k < kF; ++k) v[k] = d[k][i];
+  store_fields<S>(P, base, slot, lane, v, dz);
 }
 
 // Stores the 98 post-collision deviations: direction i goes to the slot and cell of
