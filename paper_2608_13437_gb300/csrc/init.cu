@@ -207,14 +207,16 @@ __device__ __forceinline__ float equilibrium_dev(const Equilibrium& q, int k, in
 // with slots 2, 4, 6 one cell further along +x, +y, +z) and the held-x ghosts, and
 // set *bad (if given) when a cell's state is not finite. Blocks of whole warps, so a
 // warp covers one 32-cell tile. A direction's 14 values are formed as they are stored, so
-// four blocks fit an SM (three with all 98 values at once; five spill), and the maxima go
-// to memory only where they exceed what is there: one atomic per warp and field, all on 14
-// words, was half of a small domain's time. From five fields, both passes where there are
-// two: 64^3 FP16 240 -> 125 us, 128^3 FP16 520 -> 335, 128^3 FP32 twist 370 -> 280, 512^3
-// FP32 11.9 -> 9.6 ms, which is 52.6 GB written and 2.7 read.
-constexpr int kInitBlocks = 4;
-template <typename S>
-__global__ void __launch_bounds__(128, kInitBlocks) k_init(const DomainConst P, const InitSpec sp, int mode,
+// four blocks fit an SM (three with all 98 values at once; five spill), and eight of the
+// maxima's pass, which waits for the fields of its next cell and has nothing to store. The
+// maxima are reduced per block and go to memory only where they exceed what is there: one
+// atomic per warp and field, all on 14 words, was half of a small domain's time. From five
+// fields, both passes where there are two: 64^3 FP16 240 -> 116 us, 128^3 FP16 520 -> 290,
+// 256^3 FP16 2270 -> 1360, 128^3 FP32 twist 370 -> 270, 512^3 FP32 11.9 -> 9.6 ms, which
+// is 52.6 GB written and 2.7 read.
+constexpr int kInitBlocks[2] = {8, 4};
+template <typename S, int MODE>
+__global__ void __launch_bounds__(128, kInitBlocks[MODE]) k_init(const DomainConst P, const InitSpec sp,
                                               S* __restrict__ pop, float* __restrict__ ghost,
                                               unsigned* __restrict__ maxbits,
                                               unsigned* __restrict__ bad) {
@@ -235,7 +237,7 @@ __global__ void __launch_bounds__(128, kInitBlocks) k_init(const DomainConst P, 
     initial_cell(P, sp, x, y, z, cell, c);
     Equilibrium q;
     equilibrium_of(P, c, q);
-    if (mode == 0) {
+    if constexpr (MODE == 0) {
 #pragma unroll
       for (int k = 0; k < kF; ++k)
 #pragma unroll
@@ -271,15 +273,19 @@ __global__ void __launch_bounds__(128, kInitBlocks) k_init(const DomainConst P, 
         for (int k = 0; k < kF; ++k) ghost[(1LL * kF + k) * planes + plane] = equilibrium_dev(q, k, 2);
     }
   }
-  if (mode == 0) {
+  if constexpr (MODE == 0) {
+    // order of non-negative floats = order of their bits
+    __shared__ unsigned most[kF];
+    if (threadIdx.x < kF) most[threadIdx.x] = 0;
+    __syncthreads();
 #pragma unroll
     for (int k = 0; k < kF; ++k) {
-      float m = mx[k];
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      // order of non-negative floats = order of their bits; the word only ever grows
-      if ((threadIdx.x & 31) == 0 && m > 0.0f && __float_as_uint(m) > __ldcg(&maxbits[k]))
-        atomicMax(&maxbits[k], __float_as_uint(m));
+      const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(mx[k]));
+      if ((threadIdx.x & 31) == 0) atomicMax(&most[k], m);
     }
+    __syncthreads();
+    if (threadIdx.x < kF && most[threadIdx.x] > __ldcg(&maxbits[threadIdx.x]))  // it only grows
+      atomicMax(&maxbits[threadIdx.x], most[threadIdx.x]);
   }
 }
 
@@ -350,15 +356,16 @@ __global__ void __launch_bounds__(kMeanThreads) k_field_sums_final(const double*
   if (threadIdx.x < 2) sums[threadIdx.x] = sh[threadIdx.x][0];
 }
 
-// Blocks of k_init. The maxima: the resident blocks, so that each warp reduces once (64^3:
-// 100 -> 82 us for both passes of a TGV with 32 blocks per SM before). Populations from a
-// closed form: a block per 128 cells, which the hardware starts in order, so the writes
-// stay close together (512^3 esoteric twist: 8.81 -> 6.94 ms). Populations from fields: 32
-// blocks per SM that stride over the cells; the reads of the next cells start while the
-// last writes drain (512^3: 10.65 -> 9.63 ms).
+// Blocks of k_init. The maxima: the resident blocks, so that each reduces once (64^3 TGV,
+// both passes: 100 us with 32 blocks per SM, 82 with the resident ones, 69 with eight of
+// those per SM and one reduction per block). Populations from a closed form: a block per
+// 128 cells, which the hardware starts in order, so the writes stay close together (512^3
+// esoteric twist: 8.81 -> 6.94 ms). Populations from fields: 32 blocks per SM that stride
+// over the cells; the reads of the next cells start while the last writes drain (512^3:
+// 10.65 -> 9.63 ms).
 int init_grid(long long n, int block, int mode, int kind) {
   const long long full = (n + block - 1) / block;
-  const long long most = mode == 0 ? 152LL * kInitBlocks : (kind < 2 ? (1LL << 30) : 152LL * 32);
+  const long long most = mode == 0 ? 152LL * kInitBlocks[0] : (kind < 2 ? (1LL << 30) : 152LL * 32);
   return (int)std::max<long long>(1, std::min(full, most));
 }
 
@@ -435,10 +442,15 @@ cudaError_t launch_init(const DomainConst& P, int store, const InitSpec& spec, i
                         float* ghost, unsigned* maxbits, unsigned* bad, cudaStream_t s) {
   const int block = 128;
   const int grid = init_grid(P.ncell, block, mode, spec.kind);
+  auto launch = [&](auto* p) {
+    using S = std::remove_pointer_t<decltype(p)>;
+    if (mode == 0) k_init<S, 0><<<grid, block, 0, s>>>(P, spec, p, ghost, maxbits, bad);
+    else k_init<S, 1><<<grid, block, 0, s>>>(P, spec, p, ghost, maxbits, bad);
+  };
   switch (store) {
-    case 0: k_init<float><<<grid, block, 0, s>>>(P, spec, mode, static_cast<float*>(pop), ghost, maxbits, bad); break;
-    case 1: k_init<__half><<<grid, block, 0, s>>>(P, spec, mode, static_cast<__half*>(pop), ghost, maxbits, bad); break;
-    default: k_init<__nv_bfloat16><<<grid, block, 0, s>>>(P, spec, mode, static_cast<__nv_bfloat16*>(pop), ghost, maxbits, bad); break;
+    case 0: launch(static_cast<float*>(pop)); break;
+    case 1: launch(static_cast<__half*>(pop)); break;
+    default: launch(static_cast<__nv_bfloat16*>(pop)); break;
   }
   return cudaGetLastError();
 }
