@@ -9,6 +9,7 @@
 // central differences of u from the field. Each pass writes one record per block
 // (warp shuffles, then shared memory) and the last block of pass B to finish reduces the
 // records in a fixed order, so results are reproducible run to run.
+#include <algorithm>
 #include <atomic>
 
 #include "diag_device.cuh"
@@ -156,31 +157,41 @@ __device__ __forceinline__ void ldv(const float* p, float (&o)[kCells]) {
 // kBlockB threads: thread (j, s) folds records s, s + 8, ... of quantity j, then the 8
 // slices are added in order. The reference density and energy are added back once per
 // cell at the end, the maximum Mach number is the root of the maximum of Mach^2 and the
-// maximum CFL number the maximum speed / c. Latency-bound (a few hundred KB): as a kernel
-// of its own over a fixed 1216 records, with every thread holding all 15 quantities and
-// an FP64 tree over 256 threads, it took 20 us whatever the domain.
-__device__ void diag_final(const DomainConst& P, const double* __restrict__ pa, int nblocks_a,
+// maximum CFL number the maximum speed / c. Bound by the trips to the L2 (a few hundred
+// KB), so a thread has 16 loads in flight and folds them in order; one load at a time took
+// 48 us for the 1216 records of a step with diagnostics and 21 us for the 304 of pass A (a
+// kernel of its own over 1216 records, with every thread holding all 15 quantities and an
+// FP64 tree over 256 threads, 20 us). Not inlined: its registers cost the march of pass B
+// 8 % (512^3: 500 us with it inlined, 459 so; 468 for pass B and that kernel).
+__device__ __noinline__ void diag_final(const DomainConst& P, const double* __restrict__ pa, int nblocks_a,
                            const double* __restrict__ pb, int nblocks_b, double* __restrict__ out) {
-  constexpr int kN = kDiagA + 2, kSlices = kBlockB / 16;
+  constexpr int kN = kDiagA + 2, kSlices = kBlockB / 16, kBatch = 16;
   __shared__ double sh[kSlices][16];
   const int j = threadIdx.x & 15, sl = threadIdx.x >> 4;
-  if (j < 9 || j >= kDiagA) {  // sums
-    double r = 0.0;
-    if (j < 9) {
-      for (int b = sl; b < nblocks_a; b += kSlices) r += __ldcg(pa + (long long)b * kDiagA + j);
-    } else if (j < kN) {
-      for (int b = sl; b < nblocks_b; b += kSlices) r += __ldcg(pb + (long long)b * 2 + (j - kDiagA));
+  const bool of_a = j < kDiagA, extremum = j >= 9 && of_a, largest = j < 11;
+  const double* const from = of_a ? pa + j : pb + (j - kDiagA);
+  const int step = of_a ? kDiagA : 2, n = of_a ? nblocks_a : (j < kN ? nblocks_b : 0);
+  // sums fold in FP64; extrema are FP32 values held in FP64
+  const double none = extremum ? (largest ? -INFINITY : INFINITY) : 0.0;
+  double r = none;
+  for (int b = sl; b < n; b += kBatch * kSlices) {
+    double v[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int at = b + q * kSlices;
+      v[q] = at < n ? __ldcg(from + (long long)at * step) : none;
     }
-    sh[sl][j] = r;
-  } else {  // extrema: FP32 values held in FP64
-    const bool mx = j < 11;
-    float r = mx ? -INFINITY : INFINITY;
-    for (int b = sl; b < nblocks_a; b += kSlices) {
-      const float v = (float)__ldcg(pa + (long long)b * kDiagA + j);
-      r = mx ? fmaxf(r, v) : fminf(r, v);
+    if (extremum) {
+      float m = (float)r;
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) m = largest ? fmaxf(m, (float)v[q]) : fminf(m, (float)v[q]);
+      r = m;
+    } else {
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) r += v[q];
     }
-    sh[sl][j] = r;
   }
+  sh[sl][j] = r;
   __syncthreads();
   if (threadIdx.x < kN) {
     const bool sum = j < 9 || j >= kDiagA, mx = j < 11;
@@ -579,7 +590,9 @@ cudaError_t launch_diag_records(const DomainConst& P, const float* rec, long lon
                                 cudaStream_t s) {
   double* pa = partials;
   double* pb = partials + (long long)kDiagBlocks * kDiagA;
-  const int blocks = blocks_for(nrec);
+  // 4 blocks per SM: 512^3 (4.2 M records) 63-70 us with 8, 56 with 4, 79 with 2; and the
+  // last block of pass B has half the records to fold
+  const int blocks = std::min(blocks_for(nrec), kDiagBlocks / 2);
   k_diag_records<<<blocks, kBlock, 0, s>>>(rec, nrec, pa, ticket_of(out16));
   launch_b(P, ufield, pa, blocks, pb, ticket_of(out16), out16, s);
   return cudaGetLastError();
