@@ -685,10 +685,15 @@ lbm_status lbm_step(lbm_handle* h, int n) {
   }
   while (use_resident(h, n)) {
     const int m = n < kResidentMostSteps ? n : kResidentMostSteps;
-    LBM_CUDA(launch_resident(h->P, h->res, h->prm.store, (int)(h->step & 1), h->pop, h->ghost, h->flag,
-                             h->res_mem,
-                             reinterpret_cast<unsigned*>(static_cast<char*>(h->res_mem) + h->res_inbox),
-                             m, h->stream));
+    const cudaError_t e = launch_resident(
+        h->P, h->res, h->prm.store, (int)(h->step & 1), h->pop, h->ghost, h->flag, h->res_mem,
+        reinterpret_cast<unsigned*>(static_cast<char*>(h->res_mem) + h->res_inbox), m, h->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer SMs for this process than the device has
+      cudaGetLastError();
+      h->res_on = false;
+      break;
+    }
+    LBM_CUDA(e);
     h->step += m;
     n -= m;
   }
