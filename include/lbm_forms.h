@@ -1,0 +1,25 @@
+/*
+ * lbm_forms.h -- the form in which lbm_step runs the steps of a domain (no counterpart in
+ * the paper).
+ */
+#ifndef LBM_FORMS_H_
+#define LBM_FORMS_H_
+
+#include "lbm.h"
+
+#ifdef __cplusplus
+extern "C" {
+#endif
+
+/* Failure-detection test hook. In the next launch that takes many steps of a small domain
+ * (lbm_step), block `block` does nothing, and a wait of the others gives up after `polls`
+ * tries (about half a microsecond each, rounded up to 1024) instead of about a second. Its neighbours' waits
+ * run out; nothing faults or hangs. The next synchronising call then returns
+ * LBM_E_TIMEOUT, after which lbm_step refuses to run until a re-init. LBM_E_INVAL if the
+ * domain takes one launch per step, for a block it does not have or polls < 1. */
+lbm_status lbm_test_stall_resident(lbm_handle* h, int block, int polls);
+
+#ifdef __cplusplus
+}
+#endif
+#endif /* LBM_FORMS_H_ */

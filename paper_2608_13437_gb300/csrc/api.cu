@@ -11,6 +11,7 @@
 #include "api_common.h"
 #include "host_pages.h"
 #include "lbm_arrays.h"
+#include "lbm_forms.h"
 
 using namespace lbm;
 
@@ -196,7 +197,8 @@ struct lbm_handle {
   ResidentPlan res;
   bool res_on = false;         // the domain is small enough, and no kernel form was asked for
   void* res_mem = nullptr;
-  size_t res_inbox = 0, res_bytes = 0;
+  size_t res_inbox = 0;        // bytes; the step counts follow
+  int res_polls = kResidentPolls, res_silent = -1;  // of the next launch (test hook)
 };
 
 namespace {
@@ -306,9 +308,9 @@ void setup_resident(lbm_handle* h) {
   }
   if (!coop || !resident_plan(h->P, h->prm.store, sms, &h->res)) return;
   h->res_inbox = resident_inbox_bytes(h->res, h->prm.store);
-  h->res_bytes = h->res_inbox + sizeof(unsigned) * (size_t)h->res.blocks();
-  if (cudaMalloc(&h->res_mem, h->res_bytes) != cudaSuccess ||
-      cudaMemset(h->res_mem, 0, h->res_bytes) != cudaSuccess ||
+  const size_t bytes = h->res_inbox + sizeof(unsigned) * (size_t)h->res.blocks();
+  if (cudaMalloc(&h->res_mem, bytes) != cudaSuccess ||
+      cudaMemset(h->res_mem, 0, bytes) != cudaSuccess ||
       cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
     cudaGetLastError();
     if (h->res_mem) cudaFree(h->res_mem);
@@ -361,8 +363,6 @@ void set_reference(lbm_handle* h, double rho_ref, double E_ref) {
 // Runs both init passes for an initial state: Q_ref must be set beforehand.
 lbm_status run_init(lbm_handle* h, InitSpec& sp) {
   reset_scales(h);
-  if (h->stalled && h->res_mem)  // blocks that gave up waiting left their step counts apart
-    LBM_CUDA(cudaMemsetAsync(h->res_mem, 0, h->res_bytes, h->stream));
   if (h->prm.store == LBM_STORE_F16) {
     LBM_CUDA(cudaMemsetAsync(h->maxbits, 0, kF * sizeof(unsigned), h->stream));
     LBM_CUDA(launch_init(h->P, h->prm.store, sp, 0, h->pop, h->ghost, h->maxbits, nullptr, h->stream));
@@ -685,15 +685,18 @@ lbm_status lbm_step(lbm_handle* h, int n) {
   }
   while (use_resident(h, n)) {
     const int m = n < kResidentMostSteps ? n : kResidentMostSteps;
+    const ResidentRun run{m, h->res_polls, h->res_silent};
     const cudaError_t e = launch_resident(
         h->P, h->res, h->prm.store, (int)(h->step & 1), h->pop, h->ghost, h->flag, h->res_mem,
-        reinterpret_cast<unsigned*>(static_cast<char*>(h->res_mem) + h->res_inbox), m, h->stream);
+        reinterpret_cast<unsigned*>(static_cast<char*>(h->res_mem) + h->res_inbox), run, h->stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {  // fewer SMs for this process than the device has
       cudaGetLastError();
       h->res_on = false;
       break;
     }
     LBM_CUDA(e);
+    h->res_polls = kResidentPolls;
+    h->res_silent = -1;
     h->step += m;
     n -= m;
   }
@@ -1157,6 +1160,16 @@ lbm_status lbm_test_skip_copy(lbm_handle* h) {
   if (!h) return fail(LBM_E_INVAL, "handle is NULL");
   if (h->variant < kFirstStagedVariant) return fail(LBM_E_INVAL, "the kernel form is not staged");
   h->skip_next_copy = true;
+  return LBM_OK;
+}
+
+lbm_status lbm_test_stall_resident(lbm_handle* h, int block, int polls) {
+  if (!h) return fail(LBM_E_INVAL, "handle is NULL");
+  if (!h->res_on) return fail(LBM_E_INVAL, "the domain takes one launch per step");
+  if (block < 0 || block >= h->res.blocks() || polls < 1 || polls > kResidentPolls)
+    return fail(LBM_E_INVAL, "block must be below %d, polls 1 to %d", h->res.blocks(), kResidentPolls);
+  h->res_silent = block;
+  h->res_polls = (polls + kResidentPollsPerLook - 1) / kResidentPollsPerLook * kResidentPollsPerLook;
   return LBM_OK;
 }
 

@@ -121,9 +121,18 @@ bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R);
 // Bytes of the bricks' inboxes (zeroed before the first launch; so are the epochs, one
 // word per block).
 size_t resident_inbox_bytes(const ResidentPlan& R, int store);
+// Tries of one wait before a block gives up: each is a trip through the L2 (about half a
+// microsecond), so about a second.
+constexpr int kResidentPolls = 1 << 21;
+constexpr int kResidentPollsPerLook = 1024;  // between two looks whether another block has given up
+struct ResidentRun {
+  int steps;
+  int polls;   // tries of one wait, a multiple of kResidentPollsPerLook
+  int silent;  // a block that does nothing (failure-detection test), or -1
+};
 cudaError_t launch_resident(const DomainConst& P, const ResidentPlan& R, int store, int parity,
                             void* pop, const float* ghost, unsigned* flag, void* inbox,
-                            unsigned* epochs, int steps, cudaStream_t s);
+                            unsigned* epochs, const ResidentRun& run, cudaStream_t s);
 
 // SMs of the current device (looked up once per device).
 int sm_count();

@@ -24,10 +24,13 @@
 //     which they send after they have loaded theirs, and a location is loaded and stored by
 //     one brick and its direct neighbours along that population's axis alone.
 //   * Launched cooperatively (every block resident, or the launch fails). A poll gives up
-//     after a bounded number of tries; the block then sets flag bit 2 and returns without
-//     storing, its neighbours run out the same way, and the host reports LBM_E_TIMEOUT.
+//     after a bounded number of tries, or soon after another block has; the block then sets
+//     flag bit 2 and returns without storing, launches that find the bit set do nothing, and
+//     the host reports LBM_E_TIMEOUT.
 //   * Tags go on from each block's own step count in device memory, so a launch may be
-//     repeated (also by a graph) without the host's knowledge of it.
+//     repeated (also by a graph) without the host's knowledge of it. A block that gives up or
+//     does nothing counts the launch's steps all the same, so the counts stay equal and
+//     nothing that a failed launch leaves in an inbox passes for a later step's.
 #include <algorithm>
 
 #include "lbm_internal.h"
@@ -148,9 +151,11 @@ __device__ __forceinline__ uint4 packet_load(const uint4* p) {
   return make_uint4((unsigned)lo, (unsigned)(lo >> 32), (unsigned)hi, (unsigned)(hi >> 32));
 }
 
-// Tries of one poll before a block gives up: each is a trip through the L2 (about half a
-// microsecond), so about a second.
-constexpr int kMaxPolls = 1 << 21;
+__device__ __forceinline__ bool gave_up(const unsigned* flag) {
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
+  return (v & 2u) != 0;
+}
 
 // Exchange buffers of a block: two where 200 KB of shared memory hold them, which saves a
 // barrier per step.
@@ -167,11 +172,13 @@ template <typename S, bool SR, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
     k_resident(const DomainConst P, const ResidentPlan R, S* __restrict__ pop,
                const float* __restrict__ ghost, unsigned* __restrict__ flag,
-               uint4* __restrict__ inbox, unsigned* __restrict__ epochs, int parity0, int steps) {
+               uint4* __restrict__ inbox, unsigned* __restrict__ epochs, int parity0,
+               const ResidentRun run) {
   using V4 = typename Codec<S>::V4;
   using V2 = typename Codec<S>::V2;
   constexpr int NW = Words<S>::n, NP = Words<S>::packets;
   extern __shared__ __align__(16) unsigned char smem[];
+  const int steps = run.steps;
   const int T = blockDim.x, tid = threadIdx.x;
   // exchange buffers (one, or two for even and odd tags), the rest populations of the last
   // step, and the table of the packet sets that arrive from outside
@@ -238,11 +245,16 @@ __global__ void __launch_bounds__(MAXT, 1)
       n_in += 2 * w[u] * w[v];
     }
   }
-  __syncthreads();
+  const unsigned epoch = epochs[blockIdx.x];
+  // Nothing is done with the incomplete state that a launch before this one left, nor by a
+  // block that is to fail: its neighbours wait in vain.
+  if (__syncthreads_or(tid == 0 && (gave_up(flag) || (int)blockIdx.x == run.silent))) {
+    if (tid == 0) epochs[blockIdx.x] = epoch + (unsigned)steps;
+    return;
+  }
 
   float d[kF][kQ];
   const CellIndex c = make_index(P, x, y, z);
-  const unsigned epoch = epochs[blockIdx.x];
   if (active) {
     if (parity0) load_cell<1, false, S>(P, pop, nullptr, c, d);
     else load_cell<0, false, S>(P, pop, nullptr, c, d);
@@ -325,7 +337,7 @@ __global__ void __launch_bounds__(MAXT, 1)
       const uint2 in = table[e];
       const uint4* p = inbox + in.x + (tag & 1u) * (unsigned)(NP * R.sets);
       unsigned w[3 * NP];
-      for (int tries = 0;; ++tries) {
+      for (int tries = 0;;) {
         uint4 m[NP];
 #pragma unroll
         for (int q = 0; q < NP; ++q) m[q] = packet_load(p + (size_t)q * R.sets);
@@ -339,7 +351,7 @@ __global__ void __launch_bounds__(MAXT, 1)
           if (3 * q + 1 >= NW) ok = ok && m[q].y == tag;
           if (3 * q + 2 >= NW) ok = ok && m[q].z == tag;
         }
-        if (ok || dead || tries >= kMaxPolls) {
+        if (ok || dead) {
           dead = dead || !ok;
 #pragma unroll
           for (int q = 0; q < NP; ++q) {
@@ -349,13 +361,17 @@ __global__ void __launch_bounds__(MAXT, 1)
           }
           break;
         }
+        if ((++tries & (kResidentPollsPerLook - 1)) == 0) dead = tries >= run.polls || gave_up(flag);
       }
 #pragma unroll
       for (int g = 0; g < 3; ++g) s4[(in.y >> 16) * 3 * T + g * T + (in.y & 0xFFFFu)] = words4<S>(w, g);
       s2[(in.y >> 16) * T + (in.y & 0xFFFFu)] = words2<S>(w);
     }
     if (__syncthreads_or(dead)) {  // a block whose wait ran out stops here
-      if (tid == 0) atomicOr(flag, 2u);
+      if (tid == 0) {
+        atomicOr(flag, 2u);
+        epochs[blockIdx.x] = epoch + (unsigned)steps;
+      }
       return;
     }
     if (active) {
@@ -392,7 +408,7 @@ constexpr size_t smem_bytes(int threads) {
 
 template <typename S, bool SR, int MAXT>
 cudaError_t launch_threads(const DomainConst& P, const ResidentPlan& R, void* pop, const float* ghost,
-                     unsigned* flag, void* inbox, unsigned* epochs, int parity, int steps,
+                     unsigned* flag, void* inbox, unsigned* epochs, int parity, const ResidentRun& run,
                      cudaStream_t s) {
   const size_t smem = smem_bytes<S, MAXT>(R.threads);
   cudaError_t e = cudaFuncSetAttribute(k_resident<S, SR, MAXT>,
@@ -410,16 +426,16 @@ cudaError_t launch_threads(const DomainConst& P, const ResidentPlan& R, void* po
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, k_resident<S, SR, MAXT>, P, R, static_cast<S*>(pop), ghost, flag,
-                            static_cast<uint4*>(inbox), epochs, parity, steps);
+                            static_cast<uint4*>(inbox), epochs, parity, run);
 }
 
 template <typename S, bool SR>
 cudaError_t launch_t(const DomainConst& P, const ResidentPlan& R, void* pop, const float* ghost,
-                     unsigned* flag, void* inbox, unsigned* epochs, int parity, int steps,
+                     unsigned* flag, void* inbox, unsigned* epochs, int parity, const ResidentRun& run,
                      cudaStream_t s) {
   if (R.threads <= 256)
-    return launch_threads<S, SR, 256>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
-  return launch_threads<S, SR, kResidentMaxThreads>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
+    return launch_threads<S, SR, 256>(P, R, pop, ghost, flag, inbox, epochs, parity, run, s);
+  return launch_threads<S, SR, kResidentMaxThreads>(P, R, pop, ghost, flag, inbox, epochs, parity, run, s);
 }
 
 }  // namespace
@@ -473,15 +489,15 @@ size_t resident_inbox_bytes(const ResidentPlan& R, int store) {
 
 cudaError_t launch_resident(const DomainConst& P, const ResidentPlan& R, int store, int parity,
                             void* pop, const float* ghost, unsigned* flag, void* inbox,
-                            unsigned* epochs, int steps, cudaStream_t s) {
+                            unsigned* epochs, const ResidentRun& run, cudaStream_t s) {
   cudaError_t e;
-  if (store == 0) e = launch_t<float, false>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
+  if (store == 0) e = launch_t<float, false>(P, R, pop, ghost, flag, inbox, epochs, parity, run, s);
   else if (store == 1)
-    e = P.sround ? launch_t<__half, true>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s)
-                 : launch_t<__half, false>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
+    e = P.sround ? launch_t<__half, true>(P, R, pop, ghost, flag, inbox, epochs, parity, run, s)
+                 : launch_t<__half, false>(P, R, pop, ghost, flag, inbox, epochs, parity, run, s);
   else
-    e = P.sround ? launch_t<__nv_bfloat16, true>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s)
-                 : launch_t<__nv_bfloat16, false>(P, R, pop, ghost, flag, inbox, epochs, parity, steps, s);
+    e = P.sround ? launch_t<__nv_bfloat16, true>(P, R, pop, ghost, flag, inbox, epochs, parity, run, s)
+                 : launch_t<__nv_bfloat16, false>(P, R, pop, ghost, flag, inbox, epochs, parity, run, s);
   if (e != cudaSuccess) cudaGetLastError();
   return e;
 }

@@ -102,3 +102,65 @@ def test_resident_handles_on_two_streams(lbm):
         assert np.array_equal(d.populations("native"), r.populations("native"))
         r.close()
         d.close()
+
+
+@pytest.mark.parametrize("store,steps", [("f32", 40), ("f16", 5000)])
+def test_resident_wait_runs_out_and_is_reported(lbm, store, steps):
+    """Failure detection without a fault: one block does nothing, so its neighbours' bounded
+    waits run out. The next synchronising call reports LBM_E_TIMEOUT and steps are refused;
+    after a re-init the handle steps exactly like a fresh one, whether the host has seen the
+    failure in between or not. Launches queued behind the failed one end at once."""
+    import time
+    p = inputs.tgv_params(32)
+    d = lbm.Domain(p, store=store)
+    L = lbm.lib()
+    assert L.lbm_test_stall_resident(None, 0, 100) == lbm.LBM_E_INVAL
+    for block, polls in ((-1, 100), (100000, 100), (0, 0)):
+        assert L.lbm_test_stall_resident(d.handle, block, polls) == lbm.LBM_E_INVAL
+    ref = lbm.Domain(p, store=store, use_graphs=False)
+    assert L.lbm_test_stall_resident(ref.handle, 0, 100) == lbm.LBM_E_INVAL  # plain steps
+    ref.init_tgv(1.0, 1.25, 1.0)
+    ref.step(33)
+    want = ref.populations("native")
+    ref.close()
+    for synchronise in (True, False, True):
+        d.init_tgv(1.0, 1.25, 1.0)
+        d.step(9)
+        assert L.lbm_test_stall_resident(d.handle, 5, 4000) == lbm.LBM_OK
+        t0 = time.time()
+        d.step(steps)
+        if synchronise:
+            with pytest.raises(lbm.LbmError) as ei:
+                d.synchronize()
+            assert ei.value.status == lbm.LBM_E_TIMEOUT and "neighbouring block" in str(ei.value)
+            with pytest.raises(lbm.LbmError) as ei:
+                d.step(8)
+            assert ei.value.status == lbm.LBM_E_TIMEOUT
+        d.init_tgv(1.0, 1.25, 1.0)
+        assert time.time() - t0 < 1.0  # 4000 tries are a few ms
+        d.step(9)
+        d.step(24)
+        d.synchronize()
+        assert np.array_equal(d.populations("native"), want), synchronise
+    d.close()
+
+
+def test_load_after_a_wait_that_ran_out(lbm, tmp_path):
+    """A checkpoint loaded into a handle whose last launch gave up, before the host has seen
+    it, steps like the handle that was saved."""
+    p = inputs.tgv_params(32)
+    a, b = lbm.Domain(p), lbm.Domain(p)
+    for d in (a, b):
+        d.init_tgv(1.0, 1.25, 1.0)
+        d.step(9)
+    path = str(tmp_path / "ck.bin")
+    a.save(path)
+    assert lbm.lib().lbm_test_stall_resident(b.handle, 3, 4000) == lbm.LBM_OK
+    b.step(10)
+    b.load(path)
+    for d in (a, b):
+        d.step(11)
+        d.synchronize()
+    assert np.array_equal(a.populations("native"), b.populations("native"))
+    a.close()
+    b.close()
