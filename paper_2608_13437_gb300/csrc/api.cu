@@ -197,7 +197,8 @@ struct lbm_handle {
   ResidentPlan res;
   bool res_on = false;         // the domain is small enough, and no kernel form was asked for
   void* res_mem = nullptr;
-  size_t res_inbox = 0;        // bytes; the step counts follow
+  size_t res_inbox = 0, res_bytes = 0;  // the step counts follow the inboxes
+  bool res_zeroed = false;     // once, on the handle's stream, before the first launch
   int res_polls = kResidentPolls, res_silent = -1;  // of the next launch (test hook)
 };
 
@@ -308,12 +309,9 @@ void setup_resident(lbm_handle* h) {
   }
   if (!coop || !resident_plan(h->P, h->prm.store, sms, &h->res)) return;
   h->res_inbox = resident_inbox_bytes(h->res, h->prm.store);
-  const size_t bytes = h->res_inbox + sizeof(unsigned) * (size_t)h->res.blocks();
-  if (cudaMalloc(&h->res_mem, bytes) != cudaSuccess ||
-      cudaMemset(h->res_mem, 0, bytes) != cudaSuccess ||
-      cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+  h->res_bytes = h->res_inbox + sizeof(unsigned) * (size_t)h->res.blocks();
+  if (cudaMalloc(&h->res_mem, h->res_bytes) != cudaSuccess) {
     cudaGetLastError();
-    if (h->res_mem) cudaFree(h->res_mem);
     h->res_mem = nullptr;
     return;
   }
@@ -685,6 +683,10 @@ lbm_status lbm_step(lbm_handle* h, int n) {
   }
   while (use_resident(h, n)) {
     const int m = n < kResidentMostSteps ? n : kResidentMostSteps;
+    if (!h->res_zeroed) {
+      LBM_CUDA(cudaMemsetAsync(h->res_mem, 0, h->res_bytes, h->stream));
+      h->res_zeroed = true;
+    }
     const ResidentRun run{m, h->res_polls, h->res_silent};
     const cudaError_t e = launch_resident(
         h->P, h->res, h->prm.store, (int)(h->step & 1), h->pop, h->ghost, h->flag, h->res_mem,

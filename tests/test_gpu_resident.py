@@ -164,3 +164,32 @@ def test_load_after_a_wait_that_ran_out(lbm, tmp_path):
     assert np.array_equal(a.populations("native"), b.populations("native"))
     a.close()
     b.close()
+
+
+def test_creating_a_small_domain_does_not_wait_for_other_work(lbm):
+    """lbm_create returns while a kernel on the default stream is still running, and the
+    handle's steps on another stream give the plain steps' result."""
+    import torch
+    p = inputs.tgv_params(32)
+    side = torch.cuda.Stream()
+    for busy in (False, True):  # the first round fills PyTorch's memory pool
+        with torch.cuda.stream(side):
+            torch.cuda.synchronize()
+            done = torch.cuda.Event()
+            if busy:
+                with torch.cuda.stream(torch.cuda.default_stream()):
+                    torch.cuda._sleep(1 << 29)  # about a quarter of a second
+                    done.record()
+            d = lbm.Domain(p)
+            if busy:
+                assert not done.query()
+            d.init_tgv(1.0, 1.25, 1.0)
+            d.step(20)
+            d.synchronize()
+            got = d.populations("native")
+            d.close()
+    r = lbm.Domain(p, use_graphs=False)
+    r.init_tgv(1.0, 1.25, 1.0)
+    r.step(20)
+    assert np.array_equal(got, r.populations("native"))
+    r.close()
