@@ -11,6 +11,10 @@
 extern "C" {
 #endif
 
+/* Steps that the handle has taken in the form which runs many steps of a small domain in one
+ * launch (lbm_step), since lbm_create. LBM_E_INVAL for a NULL argument. */
+lbm_status lbm_resident_steps(const lbm_handle* h, long long* steps);
+
 /* Failure-detection test hook. In the next launch that takes many steps of a small domain
  * (lbm_step), block `block` does nothing, and a wait of the others gives up after `polls`
  * tries (about half a microsecond each, rounded up to 1024) instead of about a second. Its neighbours' waits

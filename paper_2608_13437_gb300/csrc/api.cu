@@ -5,7 +5,10 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "api_common.h"
@@ -198,6 +201,8 @@ struct lbm_handle {
   bool res_on = false;         // the domain is small enough, and no kernel form was asked for
   void* res_mem = nullptr;
   size_t res_inbox = 0, res_bytes = 0;  // the step counts follow the inboxes
+  int res_sms = 0;             // SMs of the device
+  long long res_cost = 0, res_steps = 0;  // nanoseconds that the plan counts with; steps taken
   bool res_zeroed = false;     // once, on the handle's stream, before the first launch
   int res_polls = kResidentPolls, res_silent = -1;  // of the next launch (test hook)
 };
@@ -206,9 +211,47 @@ namespace {
 
 constexpr int kChunkPairs = 16;  // a chunk graph holds 32 steps
 // The resident form is taken for calls of at least this many steps (a launch loads and
-// stores the whole state once); one launch of it takes at most kResidentMostSteps.
+// stores the whole state once); one launch of it takes at most kResidentMostSteps, 1 to 2 ms,
+// after which kernels that wait for its SMs on other streams get their turn.
 constexpr int kResidentLeastSteps = 8;
-constexpr int kResidentMostSteps = 4096;
+constexpr int kResidentMostSteps = 512;
+
+// The streams of the live handles with a resident plan. Launches on different streams would
+// compete for the SMs, so lbm_step weighs their number (resident_pays); results do not
+// depend on the form.
+class SmallDomains {
+ public:
+  void add(const lbm_handle* h) {
+    std::lock_guard<std::mutex> lock(m_);
+    live_[key(h)] += 1;
+  }
+  void remove(const lbm_handle* h) {
+    std::lock_guard<std::mutex> lock(m_);
+    const auto it = live_.find(key(h));
+    if (it != live_.end() && --it->second == 0) live_.erase(it);
+  }
+  int streams(int device) {
+    std::lock_guard<std::mutex> lock(m_);
+    int n = 0;
+    for (const auto& e : live_) n += e.first.first == device;
+    return n;
+  }
+
+ private:
+  using Key = std::pair<int, const void*>;
+  static Key key(const lbm_handle* h) {
+    // one default stream whatever its name; a per-thread one may differ for every handle
+    if (h->stream == cudaStreamLegacy) return {h->device, nullptr};
+    if (h->stream == cudaStreamPerThread) return {h->device, h};
+    return {h->device, h->stream};
+  }
+  std::mutex m_;
+  std::map<Key, int> live_;
+};
+SmallDomains& small_domains() {
+  static SmallDomains* all = new SmallDomains;  // never destroyed: handles may outlive main
+  return *all;
+}
 
 #define LBM_CUDA(expr)                                                                        \
   do {                                                                                        \
@@ -307,7 +350,8 @@ void setup_resident(lbm_handle* h) {
     cudaGetLastError();
     return;
   }
-  if (!coop || !resident_plan(h->P, h->prm.store, sms, &h->res)) return;
+  if (!coop || !resident_plan(h->P, h->prm.store, sms, &h->res, &h->res_cost)) return;
+  h->res_sms = sms;
   h->res_inbox = resident_inbox_bytes(h->res, h->prm.store);
   h->res_bytes = h->res_inbox + sizeof(unsigned) * (size_t)h->res.blocks();
   if (cudaMalloc(&h->res_mem, h->res_bytes) != cudaSuccess) {
@@ -315,13 +359,24 @@ void setup_resident(lbm_handle* h) {
     h->res_mem = nullptr;
     return;
   }
+  try {
+    small_domains().add(h);
+  } catch (...) {  // host memory: the plain kernel serves
+    cudaFree(h->res_mem);
+    h->res_mem = nullptr;
+    return;
+  }
   h->res_on = true;
 }
 
 // Whether the next n steps go through the resident form: not on a stream under capture,
-// where lbm_step answers as the graph replay does.
+// where lbm_step answers as the graph replay does, nor where too many streams have small
+// domains to step.
 bool use_resident(const lbm_handle* h, int n) {
   if (!h->res_on || n < kResidentLeastSteps) return false;
+  if (!resident_pays(h->P, h->prm.store, h->res_sms, h->res, h->res_cost,
+                     small_domains().streams(h->device)))
+    return false;
   cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
     cudaGetLastError();
@@ -512,7 +567,10 @@ lbm_status lbm_destroy(lbm_handle* h) {
   if (h->dout) cudaFree(h->dout);
   if (h->wrec) cudaFree(h->wrec);
   if (h->stage) cudaFree(h->stage);
-  if (h->res_mem) cudaFree(h->res_mem);
+  if (h->res_mem) {
+    small_domains().remove(h);
+    cudaFree(h->res_mem);
+  }
   if (h->hdiag) cudaFreeHost(h->hdiag);
   if (h->ev_diag) cudaEventDestroy(h->ev_diag);
   if (h->cap) cudaStreamDestroy(h->cap);
@@ -699,6 +757,7 @@ lbm_status lbm_step(lbm_handle* h, int n) {
     LBM_CUDA(e);
     h->res_polls = kResidentPolls;
     h->res_silent = -1;
+    h->res_steps += m;
     h->step += m;
     n -= m;
   }
@@ -1162,6 +1221,12 @@ lbm_status lbm_test_skip_copy(lbm_handle* h) {
   if (!h) return fail(LBM_E_INVAL, "handle is NULL");
   if (h->variant < kFirstStagedVariant) return fail(LBM_E_INVAL, "the kernel form is not staged");
   h->skip_next_copy = true;
+  return LBM_OK;
+}
+
+lbm_status lbm_resident_steps(const lbm_handle* h, long long* steps) {
+  if (!h || !steps) return fail(LBM_E_INVAL, "NULL argument");
+  *steps = h->res_steps;
   return LBM_OK;
 }
 

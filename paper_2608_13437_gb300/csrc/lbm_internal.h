@@ -115,9 +115,12 @@ struct ResidentPlan {
   int first[3]; // the first of them of each axis
   int blocks() const { return g[0] * g[1] * g[2]; }
 };
-// Chooses the bricks for `sms` blocks resident at once; false if the domain does not fit or
-// the plain kernel is faster.
-bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R);
+// Chooses the bricks for `sms` blocks resident at once, and in *cost the nanoseconds of a step
+// that the choice counts with; false if the domain does not fit or the plain kernel is faster.
+bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R, long long* cost);
+// Whether the plan still pays when small domains on `streams` streams in all may step at once.
+bool resident_pays(const DomainConst& P, int store, int sms, const ResidentPlan& R, long long cost,
+                   int streams);
 // Bytes of the bricks' inboxes (zeroed before the first launch; so are the epochs, one
 // word per block).
 size_t resident_inbox_bytes(const ResidentPlan& R, int store);

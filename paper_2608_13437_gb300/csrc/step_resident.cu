@@ -440,7 +440,18 @@ cudaError_t launch_t(const DomainConst& P, const ResidentPlan& R, void* pop, con
 
 }  // namespace
 
-bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R) {
+namespace {
+
+// Nanoseconds of a plain step, of `streams` such domains at once: launches overlap, so only
+// the part that follows the cells adds up. Fitted to 64 x 4 x 4 ... 38^3 on 1 to 12 streams;
+// within 15 % while the L2 holds the states (beyond it plain steps take up to twice as long).
+long long plain_cost(const DomainConst& P, int store, int streams) {
+  return store == 0 ? 2050 + 52 * P.ncell * streams / 1000 : 2300 + 25 * P.ncell * streams / 1000;
+}
+
+}  // namespace
+
+bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R, long long* plan_cost) {
   if (!P.collide || P.ncell > (long long)sms * kResidentMaxThreads) return false;
   const int n[3] = {P.nx, P.ny, P.nz};
   long long best = -1;
@@ -479,7 +490,24 @@ bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R) {
   // FP32: 1.6 us at 1024 x 4 x 4 (3.1), 2.95 at 32^3 (3.8), 4.1 at 38^3 (5.5), 1.95 at 16^3
   // (2.2), 2.05 at 20 x 12 x 9 (2.2); FP16 1.6 (2.8), 2.6 (3.1), 3.8 (4.6), 2.0 (2.6).
   if (best < 0) return false;
-  return store != 0 || best < 2050 + 52 * P.ncell / 1000;
+  *plan_cost = best;
+  return store != 0 || best < plain_cost(P, store, 1);
+}
+
+// A launch holds its SMs for all its steps and starts only when all its blocks fit beside those
+// of other launches, so domains on several streams take turns once the SMs are full, while
+// plain launches interleave. Microseconds for one step of every domain, plain against
+// resident: 32^3 FP32 on 1, 2, 4 streams 4.0/3.1, 5.5/6.1, 8.6/12.3, FP16 3.4/2.8, 4.5/5.4,
+// 5.6/10.8; 1024 x 4 x 4 (two fit at once) FP32 on 1, 2, 4, 8 streams 3.2/1.8, 4.2/2.1, 5.5/4.0,
+// 8.8/7.9, FP16 3.0/1.8, 3.6/2.2, 4.4/4.1, 5.8/8.1; 24^3 (two fit) FP32 on 2, 4, 6 streams
+// 4.0/2.7, 5.3/5.3, 6.2/7.9; 256 x 4 x 3 (nine fit) FP16 on 8 and 12 streams 3.5/2.3, 4.1/3.1.
+// Taking turns costs up to 1.3 times the plan's time each.
+bool resident_pays(const DomainConst& P, int store, int sms, const ResidentPlan& R, long long cost,
+                   int streams) {
+  // blocks on an SM at once: registers and shared memory of up to 256 threads
+  const int per_sm = R.threads <= 256 ? 256 / R.threads : 1;
+  const int at_once = std::max(1, sms * per_sm / R.blocks());
+  return streams <= at_once || cost * streams * 6 / (5 * at_once) < plain_cost(P, store, streams);
 }
 
 size_t resident_inbox_bytes(const ResidentPlan& R, int store) {

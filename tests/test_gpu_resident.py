@@ -193,3 +193,72 @@ def test_creating_a_small_domain_does_not_wait_for_other_work(lbm):
     r.step(20)
     assert np.array_equal(got, r.populations("native"))
     r.close()
+
+
+def resident_steps(lbm, d):
+    import ctypes
+    n = ctypes.c_longlong()
+    lbm.check(lbm.lib().lbm_resident_steps(d.handle, ctypes.byref(n)))
+    return n.value
+
+
+def _cut(shape):
+    """The cubes and tubes of this file as parameters and an initial state of their own."""
+    nx, ny, nz = shape
+    p = inputs.tgv_params(16)
+    p.update(nx=nx, ny=ny, nz=nz, dx=2 * np.pi / 40, sutherland=0, f_mu=0.3, J_min=1e-3, tau_R=0.05,
+             tau_q=0.05)
+    return p
+
+
+# shape, store, streams, whether domains on that many streams still step on the chip: launches
+# that fit beside each other, ones that take turns but are the faster form all the same, and
+# ones that would take turns at a loss
+@pytest.mark.parametrize("shape,store,streams,on_chip", [
+    ((32, 32, 32), "f32", 1, True), ((32, 32, 32), "f32", 2, False), ((32, 32, 32), "f16", 2, False),
+    ((1024, 4, 4), "f32", 2, True), ((1024, 4, 4), "f32", 4, True), ((1024, 4, 4), "f16", 8, False),
+    ((64, 4, 4), "f16", 12, True), ((38, 38, 38), "bf16", 2, False), ((24, 24, 24), "f32", 2, True)])
+def test_small_domains_on_several_streams(lbm, shape, store, streams, on_chip):
+    import torch
+    doms, refs = [], []
+    for j in range(streams):
+        s = inputs.random_smooth_state(*shape, seed=5 + j, amp=0.1)
+        fields = (s["rho"], s["ux"], s["uy"], s["uz"], s["p"])
+        with torch.cuda.stream(torch.cuda.Stream()):
+            doms.append(lbm.Domain(_cut(shape), store=store))
+            doms[-1].init_fields(*fields)
+        r = lbm.Domain(_cut(shape), store=store, use_graphs=False)
+        r.init_fields(*fields)
+        r.step(60)
+        refs.append(r.populations("native"))
+        r.close()
+    for _ in range(3):
+        for d in doms:
+            d.step(20)
+    for d, ref in zip(doms, refs):
+        assert resident_steps(lbm, d) == (60 if on_chip else 0)
+        assert np.array_equal(d.populations("native"), ref)
+    for d in doms[1:]:
+        d.close()
+    doms[0].step(20)  # the others are gone
+    assert resident_steps(lbm, doms[0]) == (80 if on_chip else 20)
+    doms[0].close()
+
+
+def test_small_domains_on_one_stream_do_not_count_twice(lbm):
+    import torch
+    p = inputs.tgv_params(32)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        doms = [lbm.Domain(p) for _ in range(3)]
+        for d in doms:
+            d.init_tgv(1.0, 1.25, 1.0)
+            d.step(600)  # more than one launch
+            assert resident_steps(lbm, d) == 600
+    a = doms[0].populations("native")
+    r = lbm.Domain(p, use_graphs=False)
+    r.init_tgv(1.0, 1.25, 1.0)
+    r.step(600)
+    assert np.array_equal(a, r.populations("native"))
+    for d in doms + [r]:
+        d.close()
