@@ -2,6 +2,8 @@
 // moments (float-float sums) and primitives as the step computes them, the sensor
 // exactly as the next step computes it, canonical population arrays in and out, and
 // raw slot planes.
+#include <type_traits>
+
 #include "diag_device.cuh"
 #include "lbm_internal.h"
 #include "step_impl.cuh"
@@ -27,8 +29,15 @@ __device__ __forceinline__ void decompose(const DomainConst& P, long long cell, 
 // even and 890 at odd parity with the general index maps and 12 warps, 649 and 680 now;
 // HBM's time for its 4.2 GB is 626. FP32 was at HBM's time and stays there). An L2 prefetch
 // of the tile a warp takes next, with a grid of resident blocks, was slower (744-860).
+// WHICH: the output, or -1 to choose at run time. Primitives need five fields only, two of the
+// four groups of a slot. Behind one set of loads the other groups were fetched too where
+// held x ends make the loads conditional, so these domains take a kernel for each output
+// (256^3 primitives, odd parity: FP32 837 -> 637 us, FP16 486 -> 377; all moments FP16 787
+// -> 704). Periodic ones share a kernel: there the loads stand together in front of the
+// choice, and with one output alone they were spread out between the sums (256^3 FP16 all
+// moments 631 -> 678 us).
 constexpr int kMomThreads = 128, kMomBlocks = 4;  // 128 registers a thread
-template <typename S, int PARITY, bool HELD, bool ROWS, bool ESO>
+template <typename S, int PARITY, bool HELD, bool ROWS, bool ESO, int WHICH>
 __global__ void __launch_bounds__(kMomThreads, kMomBlocks)
     k_moments(const DomainConst P, const S* __restrict__ pop, const float* __restrict__ ghost, int which,
               void* out, int out_f64, long long c0, long long cnt) {
@@ -40,7 +49,7 @@ __global__ void __launch_bounds__(kMomThreads, kMomBlocks)
     if (r >= cnt) continue;
     float d[kF][kQ];
     load_tile_cell<PARITY, HELD, ROWS, ESO, S>(P, pop, ghost, t0 + w, lane, d);
-    if (which == 1) {
+    if (WHICH < 0 ? which == 1 : WHICH == 1) {
       float Q[kF];
 #pragma unroll
       for (int k = 0; k < kF; ++k) {
@@ -90,8 +99,13 @@ void launch_moments_t(const DomainConst& P, int parity, const S* pop, const floa
   const unsigned grid = (unsigned)(need < most ? need : most);
   with_tile_form(P, parity, [&](auto f) {
     using F = decltype(f);
-    k_moments<S, F::parity, F::held, F::rows, F::eso>
-        <<<grid, block, 0, s>>>(P, pop, ghost, which, out, out_f64, c0, cnt);
+    auto launch = [&](auto w) {
+      k_moments<S, F::parity, F::held, F::rows, F::eso, decltype(w)::value>
+          <<<grid, block, 0, s>>>(P, pop, ghost, which, out, out_f64, c0, cnt);
+    };
+    if constexpr (!F::held) launch(std::integral_constant<int, -1>{});
+    else if (which == 1) launch(std::integral_constant<int, 1>{});
+    else launch(std::integral_constant<int, 0>{});
   });
 }
 
