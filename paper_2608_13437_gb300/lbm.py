@@ -242,8 +242,8 @@ class Domain:
         check(lib().lbm_init_riemann(self._h, axis, i_split, L, R))
 
     def init_fields(self, rho, ux, uy, uz, p, dtype=np.float64):
-        if np.dtype(dtype) in (np.float32, np.float64):
-            # each array goes to the device as it is
+        if dtype is not None and np.dtype(dtype) in (np.float32, np.float64):
+            # each array goes to the device as it is (None: the arrays' common type, below)
             arrs = [np.ascontiguousarray(np.broadcast_to(a, self.shape), dtype=dtype)
                     for a in (rho, ux, uy, uz, p)]
             ptrs = (ctypes.c_void_p * 5)(*[a.ctypes.data for a in arrs])
