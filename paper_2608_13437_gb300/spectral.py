@@ -102,7 +102,7 @@ def _dissipation_device(prim, mu, T_ref, sutherland, rho_ref, L_box):
         lbm.check(L.lbm_spectral_curl_div(zh.data_ptr(), ch.data_ptr(), wh.data_ptr(), nx, ny, nz,
                                           2 * math.pi / L_box, stream))
         w = torch.fft.ifftn(wh, dim=(1, 2, 3), norm="forward").contiguous()
-        T = prim[4].contiguous()
+        T = prim[4].contiguous().resolve_neg()  # its values are read, whatever view it is
         out = torch.empty(_DOUBLES, dtype=torch.float64, device=prim.device)
         lbm.check(L.lbm_spectral_dissipation(w.data_ptr(), T.data_ptr(), nx * ny * nz, mu, T_ref,
                                              int(bool(sutherland)), out.data_ptr(), stream))

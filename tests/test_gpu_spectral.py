@@ -56,3 +56,19 @@ def test_tensors_under_autograd_take_tensor_operations(lbm):
     _, e = spectral.energy_spectrum(u)
     e.sum().backward()
     assert torch.allclose(u.grad, u.detach() / 216, rtol=1e-9, atol=1e-12)
+
+
+@pytest.mark.parametrize("sutherland", [0, 1])
+def test_a_view_that_negates_takes_its_values(lbm, sutherland):
+    """PyTorch may hand over a tensor whose stored values are the negative ones (a view with the
+    negative bit): the result is that of the tensor itself (1e-12, as above)."""
+    import torch
+    from paper_2608_13437_gb300 import spectral
+    g = torch.Generator(device="cuda").manual_seed(3)
+    prim = torch.rand(6, 9, 10, 12, dtype=torch.float64, device="cuda", generator=g) + 0.5
+    view = torch._neg_view(-prim)
+    assert view.is_neg() and torch.equal(view, prim)
+    want = spectral.dissipation(prim, 2e-3, 0.7, sutherland, 1.1)
+    assert spectral.dissipation(view, 2e-3, 0.7, sutherland, 1.1) == pytest.approx(want, rel=1e-12)
+    assert torch.allclose(spectral.energy_spectrum(view[1:4])[1], spectral.energy_spectrum(prim[1:4])[1],
+                          rtol=1e-12, atol=0)
