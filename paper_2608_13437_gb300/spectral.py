@@ -114,7 +114,10 @@ def energy_spectrum(u, L_box=2 * math.pi):
     """(k, E(k)) over unit-width shells of |k| L; sum(E) = <|u|^2> / 2."""
     import torch
     nz, ny, nx = u.shape[1:]
-    if u.ndim == 4 and len(u) == 3 and _numbers(L_box) and _on_device(u):
+    # the shells' pass adds in any order, so runs that ask for the same bits every time take
+    # the tensor operations, which give them
+    if (u.ndim == 4 and len(u) == 3 and _numbers(L_box) and _on_device(u)
+            and not torch.are_deterministic_algorithms_enabled()):
         from . import lbm
         L = lbm.lib()
         shells = L.lbm_spectral_shell_count(nx, ny, nz)

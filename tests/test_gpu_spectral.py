@@ -72,3 +72,21 @@ def test_a_view_that_negates_takes_its_values(lbm, sutherland):
     assert spectral.dissipation(view, 2e-3, 0.7, sutherland, 1.1) == pytest.approx(want, rel=1e-12)
     assert torch.allclose(spectral.energy_spectrum(view[1:4])[1], spectral.energy_spectrum(prim[1:4])[1],
                           rtol=1e-12, atol=0)
+
+
+def test_deterministic_mode_gives_the_same_bits(lbm, monkeypatch):
+    """Under torch.use_deterministic_algorithms the shells are summed by PyTorch, whose sums then
+    come out the same every time: not by this library's pass, whose order varies."""
+    import torch
+    from paper_2608_13437_gb300 import spectral
+    u = torch.randn(3, 70, 66, 72, dtype=torch.float64, device="cuda")
+    _, loose = spectral.energy_spectrum(u)
+    L = lbm.lib()
+    monkeypatch.setattr(L, "lbm_spectral_shells", None)
+    torch.use_deterministic_algorithms(True)
+    try:
+        first, *others = [spectral.energy_spectrum(u)[1] for _ in range(4)]
+    finally:
+        torch.use_deterministic_algorithms(False)
+    assert all(torch.equal(first, e) for e in others)
+    assert torch.allclose(first, loose, rtol=1e-12, atol=0)
