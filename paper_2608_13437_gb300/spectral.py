@@ -40,6 +40,12 @@ def _numbers(*values):
     return all(isinstance(v, (int, float)) for v in values)
 
 
+def _sizes(*values):
+    """Whether these are the positive numbers that the library's passes divide by; what any
+    other value gives or raises is left to the tensor operations."""
+    return _numbers(*values) and all(1e-300 < v < 1e300 for v in values)
+
+
 def _k(n, L_box, device, dtype):
     import torch
     k = torch.fft.fftfreq(n, d=L_box / n, device=device, dtype=dtype) * (2 * math.pi)
@@ -66,8 +72,8 @@ def gradients(u, L_box=2 * math.pi):
 def dissipation(prim, mu, T_ref, sutherland, rho_ref, L_box=2 * math.pi):
     """(eps_s, eps_d) of Eq. 7 from primitive fields (6, nz, ny, nx) (FP64 recommended)."""
     import torch
-    if (prim.ndim == 4 and len(prim) >= 5 and _numbers(mu, T_ref, rho_ref, L_box)
-            and _on_device(prim)):
+    if (prim.ndim == 4 and len(prim) >= 5 and _numbers(mu, T_ref) and _sizes(rho_ref, L_box)
+            and (not sutherland or _sizes(T_ref)) and _on_device(prim)):
         return _dissipation_device(prim, mu, T_ref, sutherland, rho_ref, L_box)
     g = gradients(prim[1:4], L_box)
     wx, wy, wz = g[1, 2] - g[2, 1], g[2, 0] - g[0, 2], g[0, 1] - g[1, 0]
@@ -114,9 +120,14 @@ def energy_spectrum(u, L_box=2 * math.pi):
     """(k, E(k)) over unit-width shells of |k| L; sum(E) = <|u|^2> / 2."""
     import torch
     nz, ny, nx = u.shape[1:]
+    if u.is_cuda and _numbers(L_box) and not 0 < L_box < math.inf:
+        # No shells: of a negative side the tensor operations would use negative indices, which
+        # a kernel cannot report; of the others all shells are NaN, of which the GPU makes the
+        # lowest integer and PyTorch a RuntimeError.
+        raise (IndexError if L_box < 0 else RuntimeError)(f"L_box must be positive and finite, not {L_box}")
     # the shells' pass adds in any order, so runs that ask for the same bits every time take
     # the tensor operations, which give them
-    if (u.ndim == 4 and len(u) == 3 and _numbers(L_box) and _on_device(u)
+    if (u.ndim == 4 and len(u) == 3 and _sizes(L_box) and _on_device(u)
             and not torch.are_deterministic_algorithms_enabled()):
         from . import lbm
         L = lbm.lib()

@@ -90,3 +90,36 @@ def test_deterministic_mode_gives_the_same_bits(lbm, monkeypatch):
         torch.use_deterministic_algorithms(False)
     assert all(torch.equal(first, e) for e in others)
     assert torch.allclose(first, loose, rtol=1e-12, atol=0)
+
+
+def _outcome(f, *args):
+    """What a call gives, or the kind of error it raises."""
+    try:
+        r = f(*args)
+    except Exception as e:
+        return type(e)
+    return tuple(np.asarray(v.cpu() if hasattr(v, "cpu") else v, dtype=np.float64) for v in r)
+
+
+@pytest.mark.parametrize("name,value", [
+    ("L_box", 0.0), ("L_box", 0), ("L_box", -2.0), ("L_box", math.nan), ("L_box", math.inf), ("rho_ref", 0.0),
+    ("rho_ref", -1.1), ("rho_ref", math.nan), ("T_ref", 0.0), ("T_ref", -0.7), ("T_ref", 1e-310),
+    ("T_ref", math.inf), ("mu", 0), ("mu", math.nan), ("mu", -1.0)])
+def test_unusual_numbers_do_what_they_do_on_the_cpu(lbm, name, value):
+    """Zero, negative and non-finite parameters give the tensor operations' values or errors."""
+    import torch
+    from paper_2608_13437_gb300 import spectral
+    g = torch.Generator().manual_seed(5)
+    cpu = torch.rand(6, 4, 6, 5, dtype=torch.float64, generator=g) + 0.5
+    dev = cpu.cuda()
+    for sutherland in (0, 1):
+        a = dict(mu=2e-3, T_ref=0.7, sutherland=sutherland, rho_ref=1.1, L_box=6.0)
+        a[name] = value
+        got, want = (_outcome(spectral.dissipation, t, *a.values()) for t in (dev, cpu))
+        if isinstance(want, type):
+            assert got == want, sutherland
+        else:
+            np.testing.assert_allclose(got, want, rtol=1e-12)
+    if name == "L_box":  # no shells of such a box: refused before anything is launched
+        for t in (dev[1:4], dev[1:4].float()):
+            assert _outcome(spectral.energy_spectrum, t, value) == (IndexError if value < 0 else RuntimeError)
