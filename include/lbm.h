@@ -344,10 +344,12 @@ lbm_status lbm_load(lbm_handle* h, const char* path);
 /* ---- tuning ------------------------------------------------------------------- */
 
 /* Times the step kernel for each candidate form (variants 0 and 1 at blocks of 64
- * and 128 threads, each with L2 prefetch distances 0, 512, 1024 and 2048 tiles: at most 16 candidates; the staged variants 2-4, measured slower
- * everywhere, only through lbm_set_kernel_config) on whole step pairs with CUDA events
- * on the handle's stream, and keeps the fastest in the handle; returns it in *out if
- * out != NULL. Needs an initialised state
+ * and 128 threads, each with L2 prefetch distances 0, 512, 1024 and 2048 tiles and the one
+ * that an untuned handle of this size runs with: at most 20 candidates; the staged variants
+ * 2-4, measured slower everywhere, only through lbm_set_kernel_config) on whole step pairs
+ * with CUDA events on the handle's stream, and keeps the fastest in the handle; returns it
+ * in *out if out != NULL. One launch per step throughout: calls of lbm_step that run small
+ * domains in another form (see there) go on doing so. Needs an initialised state
  * (LBM_E_STATE otherwise); each candidate runs on the live state, so the state
  * advances by an even number of steps: re-init before the run you keep. */
 lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out);
@@ -372,7 +374,7 @@ lbm_status lbm_set_kernel_config(lbm_handle* h, int block_x, int variant);
  * storage and 0 for FP32; until this call or lbm_autotune fixes a distance, the steps
  * follow the size of the state instead of the default: none when the L2 holds the
  * populations, else 1024 tiles (16-bit) or 256 (FP32). lbm_autotune
- * chooses among 0, 512, 1024 and 2048. Populations are bit-identical with any
+ * chooses among 0, 512, 1024, 2048 and that distance. Populations are bit-identical with any
  * distance. LBM_E_INVAL for tiles < 0 or > 2^20 or a NULL handle. */
 lbm_status lbm_set_prefetch(lbm_handle* h, int tiles);
 

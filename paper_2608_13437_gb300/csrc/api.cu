@@ -1,6 +1,7 @@
 // C ABI of liblbm.so for single domains: validation, device state, CUDA-graph
 // replay of the fused step, initial states, outputs, checkpoints, autotuning.
 // The declarations and their documentation are in include/lbm.h.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -1128,10 +1129,13 @@ lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out) {
     int variant, block, prefetch;
   };
   std::vector<Cand> cands;
+  std::vector<int> distances = {0, 512, 1024, 2048};
+  if (std::find(distances.begin(), distances.end(), h->pf_auto) == distances.end())
+    distances.push_back(h->pf_auto);  // what an untuned handle of this size runs with
   for (int v : {0, 1})
     for (int b : {64, 128})
       if (b <= 32 * ((h->P.nx + 31) / 32) || b == 64)
-        for (int pf : {0, 512, 1024, 2048}) cands.push_back({v, b, pf});
+        for (int pf : distances) cands.push_back({v, b, pf});
   // The staged forms (variants 2-4) are not candidates: measured slower than the plain
   // forms at every size and storage type (their shared-memory pipeline costs more
   // instructions per cell than it saves in latency, and the L2 prefetch hides the
@@ -1143,7 +1147,8 @@ lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out) {
   float best = 1e30f;
   int best_b = h->block_x, best_v = h->variant, best_grid = h->staged_grid, tried = 0;
   int best_pf = h->P.pf_tiles;
-  h->pf_chosen = true;
+  const bool chosen_before = h->pf_chosen;
+  h->pf_chosen = true;  // the trials run with the candidate's distance
   cudaError_t err = cudaSuccess;
   for (const Cand& c : cands) {
     int grid = 0;
@@ -1185,6 +1190,7 @@ lbm_status lbm_autotune(lbm_handle* h, int pairs_per_trial, lbm_tune_t* out) {
   h->variant = best_v;
   h->staged_grid = best_grid;
   h->P.pf_tiles = best_pf;
+  h->pf_chosen = chosen_before || tried > 0;
   h->graphs_valid = false;
   if (err != cudaSuccess) return fail(LBM_E_CUDA, "autotune failed: %s", cudaGetErrorString(err));
   unsigned flag = 0;

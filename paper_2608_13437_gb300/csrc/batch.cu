@@ -680,6 +680,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int steps_per_trial, int* tile_cells
   if (!b->initialized) return fail(LBM_E_STATE, "autotune needs an initialised batch");
   if (steps_per_trial < 2) steps_per_trial = 8;
   steps_per_trial += steps_per_trial & 1;  // whole pairs keep the parity
+  const bool chosen_before = b->pf_chosen;
+  if (!b->pf_chosen && b->in_l2) b->prefetch_tiles = 0;  // the distance in effect
   b->pf_chosen = true;
   const int items[] = {1, 2, 4, 8, 16, 32};  // at most 32: one tile record per lane
   const int blocks[] = {64, 128};
@@ -742,7 +744,13 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int steps_per_trial, int* tile_cells
   b->prefetch_tiles = best_pf;
   cudaEventDestroy(a);
   cudaEventDestroy(e);
-  if (st != LBM_OK) return st;
+  if (st != LBM_OK) {
+    if (!chosen_before) {  // no distance was found: back to the defaults
+      b->pf_chosen = false;
+      b->prefetch_tiles = b->store == LBM_STORE_F32 ? 0 : kDefaultPrefetch16;
+    }
+    return st;
+  }
   lbm_status s = size_grid(b);
   if (s != LBM_OK) return s;
   if (tile_cells) *tile_cells = best_i * kTile;
