@@ -151,8 +151,10 @@ typedef struct {
                                memory by bulk asynchronous copies, a persistent grid of
                                4-warp blocks: 2 stages per warp with <= 170 registers (2),
                                2 stages with <= 128 (3), 3 stages with <= 170 (4) */
-  int prefetch_tiles;       /* L2 prefetch distance of variants 0 and 1 (see
-                               lbm_set_prefetch); 0 = off */
+  int prefetch_tiles;       /* L2 prefetch distance of variants 0 and 1 as set or tuned, or the
+                               storage type's default while it is neither (see
+                               lbm_set_prefetch; lbm_prefetch_in_effect in lbm_forms.h says
+                               what the steps use); 0 = off */
   int device;               /* CUDA device ordinal the handle is bound to (see lbm_create) */
 } lbm_info_t;
 

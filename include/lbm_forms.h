@@ -11,6 +11,12 @@
 extern "C" {
 #endif
 
+/* L2 prefetch distance in tiles that the plain step kernel of this handle runs with: the one
+ * that lbm_set_prefetch or lbm_autotune fixed, or the one that follows the state's size
+ * (lbm_info_t.prefetch_tiles is the storage type's default then). LBM_E_INVAL for a NULL
+ * argument. */
+lbm_status lbm_prefetch_in_effect(const lbm_handle* h, int* tiles);
+
 /* Steps that the handle has taken in the form which runs many steps of a small domain in one
  * launch (lbm_step), since lbm_create. LBM_E_INVAL for a NULL argument. */
 lbm_status lbm_resident_steps(const lbm_handle* h, long long* steps);

@@ -1230,6 +1230,12 @@ lbm_status lbm_test_skip_copy(lbm_handle* h) {
   return LBM_OK;
 }
 
+lbm_status lbm_prefetch_in_effect(const lbm_handle* h, int* tiles) {
+  if (!h || !tiles) return fail(LBM_E_INVAL, "NULL argument");
+  *tiles = step_const(h).pf_tiles;
+  return LBM_OK;
+}
+
 lbm_status lbm_resident_steps(const lbm_handle* h, long long* steps) {
   if (!h || !steps) return fail(LBM_E_INVAL, "NULL argument");
   *steps = h->res_steps;

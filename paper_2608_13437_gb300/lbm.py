@@ -96,6 +96,7 @@ _SIGNATURES = {
     "lbm_diag_static": (_IP, [_VP, ctypes.POINTER(LbmDiag)]),
     "lbm_step_diag": (_IP, [_VP, _IP, ctypes.POINTER(LbmDiag)]),
     "lbm_test_skip_copy": (_IP, [_VP]),
+    "lbm_prefetch_in_effect": (_IP, [_VP, ctypes.POINTER(_IP)]),
     "lbm_resident_steps": (_IP, [_VP, ctypes.POINTER(ctypes.c_longlong)]),
     "lbm_test_stall_resident": (_IP, [_VP, _IP, _IP]),
     "lbm_test_encode": (_IP, [_IP, _IP, _VP, _VP, _VP, ctypes.c_longlong, _VP]),

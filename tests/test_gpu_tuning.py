@@ -49,3 +49,26 @@ def test_batch_autotune_keeps_the_result(lbm, sizes, store):
         assert np.array_equal(a.moments(d), b.moments(d))
     a.close()
     b.close()
+
+
+def _in_effect(lbm, d):
+    import ctypes
+    n = ctypes.c_int(-1)
+    lbm.check(lbm.lib().lbm_prefetch_in_effect(d.handle, ctypes.byref(n)))
+    return n.value
+
+
+# untuned: none while the L2 holds the state, else 256 tiles (FP32) or 1024 (16-bit), ragged
+# rows too; the reported default is the storage type's
+@pytest.mark.parametrize("shape,store,untuned,default", [
+    ((32, 32, 32), "f32", 0, 0), ((128, 128, 128), "f32", 256, 0), ((150, 100, 60), "f32", 256, 0),
+    ((64, 64, 64), "f16", 0, 1024), ((128, 128, 128), "bf16", 1024, 1024)])
+def test_prefetch_distance_in_effect(lbm, shape, store, untuned, default):
+    assert lbm.lib().lbm_prefetch_in_effect(None, None) == lbm.LBM_E_INVAL
+    p = inputs.tgv_params(32)
+    p.update(nx=shape[0], ny=shape[1], nz=shape[2])
+    d = lbm.Domain(p, store=store)
+    assert (_in_effect(lbm, d), d.info()["prefetch_tiles"]) == (untuned, default)
+    d.set_prefetch(7)
+    assert (_in_effect(lbm, d), d.info()["prefetch_tiles"]) == (7, 7)
+    d.close()
