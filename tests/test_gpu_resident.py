@@ -262,3 +262,53 @@ def test_small_domains_on_one_stream_do_not_count_twice(lbm):
     assert np.array_equal(a, r.populations("native"))
     for d in doms + [r]:
         d.close()
+
+
+@pytest.mark.parametrize("shape,f32,bits16", [(s, True, True) for s in SHAPES] +
+                         [((16, 16, 16), False, True), ((38, 38, 41), False, False), ((64, 64, 64), False, False)])
+def test_which_domains_step_on_the_chip(lbm, shape, f32, bits16):
+    """The shapes above take the form they are there for; calls of fewer than eight steps, a
+    kernel form that was asked for and use_graphs = 0 do not (152 SMs)."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the choice is for 152 SMs")
+    for store, on_chip in (("f32", f32), ("f16", bits16), ("bf16", bits16)):
+        for direct, form in ((False, False), (True, False), (False, True)):
+            d = lbm.Domain(_cut(shape), store=store, use_graphs=not direct)
+            if form:
+                d.set_kernel_config(64, 0)
+            d.init_fields(1.0, 0.1, 0.0, 0.0, 1.0)
+            d.step(7)
+            assert resident_steps(lbm, d) == 0
+            d.step(8)
+            assert resident_steps(lbm, d) == (8 if on_chip and not direct and not form else 0), store
+            d.close()
+
+
+# above the size limit of the resident form, below it with a kernel form asked for, held x ends
+@pytest.mark.parametrize("shape,held,form", [((64, 64, 64), 0, None), ((32, 32, 32), 0, (64, 0)),
+                                             ((40, 9, 5), 0, (32, 1)), ((128, 6, 4), 1, (64, 0)),
+                                             ((1024, 8, 8), 1, None)])
+@pytest.mark.parametrize("store", ["f32", "f16", "bf16"])
+def test_graph_replays_equal_direct_launches(lbm, shape, held, form, store):
+    """The graphs of two and of 32 steps, with single steps before and after, against one launch
+    per step: bit for bit, both streaming maps."""
+    nx, ny, nz = shape
+    for streaming in (0, 1):
+        p = dict(inputs.sod_params(64), nx=nx, ny=ny, nz=nz) if held else _cut(shape)
+        p["streaming"] = streaming
+        s = inputs.random_smooth_state(nx, ny, nz, seed=21, amp=0.1)
+        got = []
+        for graphs in (True, False):
+            d = lbm.Domain(p, store=store, use_graphs=graphs)
+            if form:
+                d.set_kernel_config(*form)
+            d.init_fields(s["rho"], s["ux"], s["uy"], s["uz"], s["p"])
+            d.step(1)
+            d.step(70)  # odd parity: one step, two replays of 32, two of 2, one step
+            assert resident_steps(lbm, d) == 0
+            d.step(33)
+            got.append(d.populations("native"))
+            d.close()
+        assert np.isfinite(got[0].view(np.float32 if store == "f32" else np.uint16).astype(np.float64)).all()
+        assert np.array_equal(*got), streaming
