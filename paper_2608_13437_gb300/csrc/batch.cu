@@ -436,7 +436,7 @@ lbm_status lbm_batch_create(int n, const lbm_params* params, lbm_batch** out) {
   }
   if (cudaMemcpy(b->d_pops, ptrs.data(), sizeof(void*) * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(b->d_tiles, tiles.data(), sizeof(uint2) * tiles.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(b->flag, 0, 64) != cudaSuccess || cudaMemset(b->d_counter, 0, 64) != cudaSuccess)
+      cudaMemset(b->flag, 0, 64) != cudaSuccess)
     return cleanup(fail(LBM_E_CUDA, "batch table upload failed"));
   int l2 = 0;
   if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, b->device) == cudaSuccess)
@@ -517,6 +517,8 @@ lbm_status lbm_batch_init_tgv(lbm_batch* b, const double* U0, const double* M0, 
   lbm_status s = upload_consts(b);
   if (s != LBM_OK) return s;
   LBM_CUDA(cudaMemsetAsync(b->flag, 0, sizeof(unsigned), b->stream));
+  // in order with the launches that use it; they leave it at zero
+  LBM_CUDA(cudaMemsetAsync(b->d_counter, 0, 64, b->stream));
   LBM_CUDA(cudaStreamSynchronize(b->stream));
   b->step = 0;
   b->initialized = true;
