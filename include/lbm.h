@@ -279,7 +279,8 @@ lbm_status lbm_synchronize(lbm_handle* h);
  * float-float sum (about 48 significant bits) of the seven populations and the
  * reference; the primitives are exactly the step's own (its FP32 sums and closure).
  * Synchronises when dst is on the host (through a device staging buffer the handle
- * keeps, of at most 256 MB, allocated on first use). */
+ * keeps, of at most 256 MB, allocated on first use and given back when another call on the
+ * handle finds the device full). */
 lbm_status lbm_moments(lbm_handle* h, int which, void* dst, int dst_on_device, int dtype);
 
 /* Sensor of the current state, [3][z][y][x]: theta = div u (physical units),
@@ -323,7 +324,8 @@ lbm_status lbm_step_diag(lbm_handle* h, int n, lbm_diag_t* out);
 lbm_status lbm_diag_static(lbm_handle* h, lbm_diag_t* out);
 
 /* Canonical populations [k][i][z][y][x] in `dtype`: F64/F32 = the physical f
- * (decoded), NATIVE = the stored bits. */
+ * (decoded), NATIVE = the stored bits. Pageable host arrays go through the staging buffer
+ * that lbm_moments describes, in smaller pieces where the device has no room for 256 MB. */
 lbm_status lbm_populations_get(lbm_handle* h, void* dst, int dst_on_device, int dtype);
 
 /* Replaces the state with canonical populations in `dtype` (F64/F32 are encoded

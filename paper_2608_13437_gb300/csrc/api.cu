@@ -414,6 +414,29 @@ void set_reference(lbm_handle* h, double rho_ref, double E_ref) {
   h->E_ref = (double)h->P.E_ref;
 }
 
+// Gives the staging buffer back (the next transfer allocates it again).
+void drop_stage(lbm_handle* h) {
+  if (!h->stage) return;
+  cudaStreamSynchronize(h->stream);
+  cudaFree(h->stage);
+  h->stage = nullptr;
+  h->stage_bytes = 0;
+}
+
+// cudaMalloc for what a call needs; when the device is full the staging buffer makes room.
+template <typename T>
+bool device_alloc(lbm_handle* h, T** p, size_t bytes) {
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  if (h->stage) {
+    drop_stage(h);
+    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+    cudaGetLastError();
+  }
+  *p = nullptr;
+  return false;
+}
+
 // Runs both init passes for an initial state: Q_ref must be set beforehand.
 lbm_status run_init(lbm_handle* h, InitSpec& sp) {
   reset_scales(h);
@@ -669,10 +692,8 @@ static lbm_status init_from_fields(lbm_handle* h, const void* fields, const void
   if (mapped) {
     dev = mapped;  // page-locked: the kernels read it directly
   } else if (!src_on_device) {
-    if (cudaMalloc(&tmp, bytes) != cudaSuccess) {
-      cudaGetLastError();
+    if (!device_alloc(h, &tmp, bytes))
       return fail(LBM_E_NOMEM, "cudaMalloc of %zu staging bytes failed", bytes);
-    }
     cudaError_t e = cudaSuccess;
     const size_t part = arrays ? bytes / nfield : bytes;
     for (int j = 0; j < (arrays ? nfield : 1) && e == cudaSuccess; ++j)
@@ -798,28 +819,25 @@ lbm_status lbm_synchronize(lbm_handle* h) {
 
 // The handle's device staging buffer for transfers to and from host memory, allocated on
 // first use and kept (no allocation or implicit device synchronisation per call); at most
-// kStageBytes, replaced by a larger one when a transfer needs it.
-static lbm_status ensure_stage(lbm_handle* h, size_t bytes) {
-  if (h->stage_bytes >= bytes) return LBM_OK;
-  if (h->stage) {
-    cudaStreamSynchronize(h->stream);
-    cudaFree(h->stage);
-  }
-  h->stage = nullptr;
-  h->stage_bytes = 0;
-  if (cudaMalloc(&h->stage, bytes) != cudaSuccess) {
+// kStageBytes, replaced by a larger one when a transfer needs it. Sets *chunk to the cells
+// per staged piece of rows of cell_bytes in all: the whole domain or whole tiles, fewer where
+// the device has no room for more (down to one tile).
+static lbm_status ensure_stage(lbm_handle* h, size_t cell_bytes, long long* chunk) {
+  const long long most = (long long)(kStageBytes / cell_bytes) / kTile * kTile;
+  *chunk = most < h->ncell ? most : h->ncell;
+  for (;;) {
+    const size_t bytes = (size_t)*chunk * cell_bytes;
+    if (h->stage_bytes >= bytes) return LBM_OK;
+    drop_stage(h);
+    if (cudaMalloc(&h->stage, bytes) == cudaSuccess) {
+      h->stage_bytes = bytes;
+      return LBM_OK;
+    }
     cudaGetLastError();
     h->stage = nullptr;
-    return fail(LBM_E_NOMEM, "staging allocation failed");
+    if (*chunk <= kTile) return fail(LBM_E_NOMEM, "staging allocation failed");
+    *chunk = (*chunk / 2 + kTile - 1) / kTile * kTile;
   }
-  h->stage_bytes = bytes;
-  return LBM_OK;
-}
-
-// Cells per staged piece of rows of cell_bytes in all: whole tiles, at most kStageBytes.
-static long long stage_cells(const lbm_handle* h, size_t cell_bytes) {
-  const long long most = (long long)(kStageBytes / cell_bytes) / kTile * kTile;
-  return most < h->ncell ? most : h->ncell;
 }
 
 // Copies the staged rows [rows][cnt] of cells [c0, c0 + cnt) to the host array [rows][ncell]
@@ -864,8 +882,8 @@ lbm_status lbm_moments(lbm_handle* h, int which, void* dst, int dst_on_device, i
     if (e != cudaSuccess) return fail(LBM_E_CUDA, "moments failed: %s", cudaGetErrorString(e));
     return LBM_OK;
   }
-  const long long chunk = stage_cells(h, es * nf);
-  lbm_status st = ensure_stage(h, (size_t)chunk * es * nf);
+  long long chunk = 0;
+  lbm_status st = ensure_stage(h, es * nf, &chunk);
   if (st != LBM_OK) return st;
   cudaError_t e = cudaSuccess;
   for (long long c0 = 0; c0 < h->ncell && e == cudaSuccess; c0 += chunk) {
@@ -898,8 +916,8 @@ lbm_status lbm_sensor(lbm_handle* h, void* dst, int dst_on_device, int dtype) {
     if (e != cudaSuccess) return fail(LBM_E_CUDA, "sensor failed: %s", cudaGetErrorString(e));
     return LBM_OK;
   }
-  const long long chunk = stage_cells(h, es * 3);
-  lbm_status st = ensure_stage(h, (size_t)chunk * es * 3);
+  long long chunk = 0;
+  lbm_status st = ensure_stage(h, es * 3, &chunk);
   if (st != LBM_OK) return st;
   cudaError_t e = cudaSuccess;
   for (long long c0 = 0; c0 < h->ncell && e == cudaSuccess; c0 += chunk) {
@@ -916,10 +934,9 @@ lbm_status lbm_sensor(lbm_handle* h, void* dst, int dst_on_device, int dtype) {
 
 static lbm_status ensure_diag_scratch(lbm_handle* h) {
   if (h->ufield) return LBM_OK;
-  if (cudaMalloc(&h->ufield, sizeof(float) * 4 * (size_t)h->ncell) != cudaSuccess ||
-      cudaMalloc(&h->partials, sizeof(double) * (size_t)kDiagBlocks * (kDiagA + 2)) != cudaSuccess ||
-      cudaMalloc(&h->dout, sizeof(double) * 16) != cudaSuccess) {
-    cudaGetLastError();
+  if (!device_alloc(h, &h->ufield, sizeof(float) * 4 * (size_t)h->ncell) ||
+      !device_alloc(h, &h->partials, sizeof(double) * (size_t)kDiagBlocks * (kDiagA + 2)) ||
+      !device_alloc(h, &h->dout, sizeof(double) * 16)) {
     if (h->ufield) cudaFree(h->ufield);
     if (h->partials) cudaFree(h->partials);
     if (h->dout) cudaFree(h->dout);
@@ -996,11 +1013,8 @@ lbm_status lbm_step_diag(lbm_handle* h, int n, lbm_diag_t* out) {
     if (h->wrec) cudaFree(h->wrec);
     h->wrec = nullptr;
     h->wrec_n = 0;
-    if (cudaMalloc(&h->wrec, sizeof(float) * kDiagRecFloats * (size_t)nrec) != cudaSuccess) {
-      cudaGetLastError();
-      h->wrec = nullptr;
+    if (!device_alloc(h, &h->wrec, sizeof(float) * kDiagRecFloats * (size_t)nrec))
       return fail(LBM_E_NOMEM, "diagnostic record allocation failed");
-    }
     h->wrec_n = nrec;
   }
   if (!h->hdiag) {
@@ -1049,8 +1063,8 @@ static lbm_status pop_transfer(lbm_handle* h, void* buf, int on_device, int dtyp
     e = move(m, 0, h->ncell);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   } else {
-    const long long chunk = stage_cells(h, es * kP);
-    lbm_status st = ensure_stage(h, (size_t)chunk * es * kP);
+    long long chunk = 0;
+    lbm_status st = ensure_stage(h, es * kP, &chunk);
     if (st != LBM_OK) return st;
     for (long long c0 = 0; c0 < h->ncell && e == cudaSuccess; c0 += chunk) {
       const long long cnt = (c0 + chunk <= h->ncell) ? chunk : h->ncell - c0;
@@ -1092,10 +1106,7 @@ static lbm_status plane_transfer(lbm_handle* h, int z, int slot, void* buf, int 
   const size_t bytes = elem_size(h->prm.store) * kF * (size_t)h->prm.nx * h->prm.ny;
   void* dev = buf;
   if (!on_device) {
-    if (cudaMalloc(&dev, bytes) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(LBM_E_NOMEM, "staging allocation failed");
-    }
+    if (!device_alloc(h, &dev, bytes)) return fail(LBM_E_NOMEM, "staging allocation failed");
   }
   cudaError_t e = cudaSuccess;
   if (set && !on_device) e = cudaMemcpyAsync(dev, buf, bytes, cudaMemcpyHostToDevice, h->stream);

@@ -152,3 +152,39 @@ def test_primitives_follow_from_the_moments(lbm, shape, held, store):
             for j, w in zip((0, 1, 2, 3, 5), want):
                 assert np.abs(P[j] - w).max() <= 4e-6 * np.abs(w).max(), (j, streaming)
         d.close()
+
+
+def test_transfers_with_little_device_memory_left(lbm):
+    """With 160 MB left on the device, a domain whose transfers stage 256 MB at a time takes
+    smaller pieces, and calls that need memory of their own get what the staging buffer holds."""
+    import torch
+    shape = (96, 96, 96)  # 347 MB of populations
+    s = inputs.random_smooth_state(*shape, seed=13, amp=0.1)
+    fields = (s["rho"], s["ux"], s["uy"], s["uz"], s["p"])
+
+    def run(d):
+        d.init_fields(*fields)
+        d.step(3)
+        f = d.populations("native")
+        g = d.populations(np.float64)
+        d.init_fields(*fields)
+        d.set_populations(f, native=True)
+        return f, g, d.moments(), d.sensor(), d.diag()["sum_E"]
+
+    a = _domain(lbm, shape)
+    want = run(a)
+    a.close()
+    torch.cuda.empty_cache()
+    d = _domain(lbm, shape)
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (160 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        got = run(d)
+        d.step(5)
+        e = d.step_diag(2)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    assert e["status"] == lbm.LBM_OK
+    d.close()
+    for x, y in zip(want, got):
+        assert np.array_equal(np.asarray(x), np.asarray(y))
