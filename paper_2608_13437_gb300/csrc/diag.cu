@@ -97,11 +97,10 @@ __global__ void __launch_bounds__(kBlock) k_diag_records(const float* __restrict
 
 // Pass B: central differences of u (FP32, from the FP32 field), weighted by mu_local;
 // per-cell products in FP32, float-float sums. Work items are columns of 32 x 16 cells
-// (x by y) over kZChunk planes; a grid of resident blocks takes them in a fixed order
-// (block b: items b, b + grid, ...), so sums are reproducible. A block of 128 threads
-// marches up its column; a thread owns 4 consecutive cells of one row (128-bit shared
-// loads). u of the column
-// with a one-cell halo in x and y (wrapped periodically), and mu_local of the column,
+// (x by y) over zchunk planes (diag_b_planes); a grid of resident blocks takes them in a
+// fixed order (block b: items b, b + grid, ...), so sums are reproducible. A block of 128
+// threads marches up its column; a thread owns 4 consecutive cells of one row (128-bit
+// shared loads). u of the column with a one-cell halo in x and y (wrapped periodically), and mu_local of the column,
 // pass through a ring of kRingB planes in shared memory, filled by asynchronous copies
 // (cp.async) two planes ahead of the plane being differenced, so the DRAM reads of the
 // planes ahead are in flight while the block computes. When nx is a multiple of 32
@@ -494,7 +493,7 @@ long long diag_b_columns(const DomainConst& P) {
 // Planes per work item of pass B. A column of the whole height is one serial march, so
 // 64^3 has 8 of them for 608 resident blocks; cutting it costs two halo planes and about
 // two planes' time of set-up per piece. The number of planes that minimises rounds x
-// (planes + 4) is taken: 2 at 64^3, 4 at 128^3, 64 at 256^3. Even, so that the sums
+// (planes + 4) is taken: 2 at 64^3, 8 at 128^3, 64 at 256^3, 74 at 512^3. Even, so that the sums
 // over pairs of planes are the same for every cut.
 int diag_b_planes(const DomainConst& P, int resident) {
   const long long cols = diag_b_columns(P);

@@ -365,7 +365,8 @@ __global__ void __launch_bounds__(kMeanThreads) k_field_sums_final(const double*
 // 10.65 -> 9.63 ms).
 int init_grid(long long n, int block, int mode, int kind) {
   const long long full = (n + block - 1) / block;
-  const long long most = mode == 0 ? 152LL * kInitBlocks[0] : (kind < 2 ? (1LL << 30) : 152LL * 32);
+  const long long sms = sm_count();
+  const long long most = mode == 0 ? sms * kInitBlocks[0] : (kind < 2 ? (1LL << 30) : sms * 32);
   return (int)std::max<long long>(1, std::min(full, most));
 }
 

@@ -245,7 +245,8 @@ __global__ void k_plane(const DomainConst P, T* __restrict__ pop, int z, int slo
 
 int grid_for(long long n, int block) {
   long long g = (n + block - 1) / block;
-  if (g > 152LL * 32) g = 152LL * 32;
+  const long long most = (long long)sm_count() * 32;
+  if (g > most) g = most;
   return (int)(g < 1 ? 1 : g);
 }
 

@@ -360,15 +360,6 @@ __device__ __forceinline__ long long dst_cell(const DomainConst& P, const CellIn
   return parity ? c.nb[i] : c.own;
 }
 
-// Cell and slot from which direction i of this cell is read at `parity`.
-__device__ __forceinline__ long long read_pos(const DomainConst& P, const CellIndex& c, int parity,
-                                              int k, int i) {
-  long long cell = src_cell(P, c, parity, i);
-  if (!LBM_CHECK(P, cell >= 0 && cell < P.ntile * kTile)) cell = 0;
-  const int slot = parity ? opp(i) : i;
-  return pop_index(cell, k, slot);
-}
-
 // Held x ends: the inward population of a boundary cell comes from the ghost
 // layer, ghost[side][k][plane] (deviation, unscaled).
 __device__ __forceinline__ bool from_ghost(const DomainConst& P, const CellIndex& c, int i) {

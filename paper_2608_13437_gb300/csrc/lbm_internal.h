@@ -51,7 +51,8 @@ inline dim3 step_grid(const DomainConst& P, int block_x) {
   return dim3((unsigned)((P.ntile * kTile + block_x - 1) / block_x));
 }
 
-// Fused step: one launch per time step, grid step_grid, block_x in {32, 64, 96, 128}; variant selects the register budget (0: 170, 1: 128 registers).
+// Fused step: one launch per time step, grid step_grid, block_x in {32, 64, 96, 128};
+// variant selects the register budget (0: 170, 1: 128 registers).
 cudaError_t launch_step_f32(const DomainConst& P, int parity, void* pop, const float* ghost,
                             unsigned* flag, int block_x, int variant, cudaStream_t s);
 cudaError_t launch_step_f16(const DomainConst& P, int parity, void* pop, const float* ghost,
@@ -67,9 +68,9 @@ cudaError_t launch_step_bf16(const DomainConst& P, int parity, void* pop, const 
 // bounded wait runs out and the step reports a stalled copy).
 constexpr int kFirstStagedVariant = 2, kLastStagedVariant = 4;
 // L2 prefetch distance (tiles ahead) of the plain and batched step kernels for 16-bit
-// storage when not tuned: about half the warps resident on the GPU at once, the
-// fastest distance measured at 512^3 (FP32 storage gains nothing from it and starts
-// with 0); the largest distance accepted.
+// storage when not tuned and the L2 does not hold the state: about half the warps resident
+// on the GPU at once, the fastest distance measured at 512^3. FP32 domains beyond the L2
+// take 256 then (auto_prefetch), FP32 batches none. The largest distance accepted.
 constexpr int kDefaultPrefetch16 = 1024;
 constexpr int kMaxPrefetch = 1 << 20;
 inline bool staged_eligible(const DomainConst& P) {
@@ -107,7 +108,7 @@ inline long long step_diag_record_count(const DomainConst& P, int block_x) {
 // Several steps of a small domain in one cooperative launch, the populations in registers
 // (step_resident.cu). A plan cuts the domain into bricks of b cells, g of them along each
 // axis, one block each.
-constexpr int kResidentMaxThreads = 384;  // cells of a brick at most: 170 registers a thread
+constexpr int kResidentMaxThreads = 384;  // cells of a brick at most: 168 registers a thread
 struct ResidentPlan {
   int b[3], g[3];
   int threads;  // of a block: the brick's cells rounded up to whole warps

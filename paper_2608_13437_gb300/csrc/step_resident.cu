@@ -5,9 +5,9 @@
 // L2 for no reason but that launches end, and costs 3.1 us at 16 thousand cells, of which
 // about 1 us is the gap between two launches and most of the rest one chain of dependent
 // loads, arithmetic and stores. Here each block keeps a brick of cells for n steps, one
-// thread per cell with its 14 x 7 populations in registers (the plain step kernel's budget
-// of 170), and per step only what the lattice links carry moves: within the brick through
-// shared memory, between bricks through inboxes in global memory (the L2).
+// thread per cell with its 14 x 7 populations in registers (255 of them for bricks of up to
+// 256 cells, 168 above), and per step only what the lattice links carry moves: within the
+// brick through shared memory, between bricks through inboxes in global memory (the L2).
 //
 //   * Every directional population leaves as the words of the storage type (rounded as a
 //     plain step's store rounds it) and is decoded on arrival as a plain step's load does;
