@@ -100,10 +100,10 @@ __global__ void __launch_bounds__(kBlock) k_diag_records(const float* __restrict
 // (x by y) over zchunk planes (diag_b_planes); a grid of resident blocks takes them in a
 // fixed order (block b: items b, b + grid, ...), so sums are reproducible. A block of 128
 // threads marches up its column; a thread owns 4 consecutive cells of one row (128-bit
-// shared loads). u of the column with a one-cell halo in x and y (wrapped periodically), and mu_local of the column,
-// pass through a ring of kRingB planes in shared memory, filled by asynchronous copies
-// (cp.async) two planes ahead of the plane being differenced, so the DRAM reads of the
-// planes ahead are in flight while the block computes. When nx is a multiple of 32
+// shared loads). u of the column with a one-cell halo in x and y (wrapped periodically),
+// and mu_local of the column, pass through a ring of kRingB planes in shared memory, filled
+// by asynchronous copies (cp.async) two planes ahead of the plane being differenced, so the
+// DRAM reads of the planes ahead are in flight while the block computes. When nx is a multiple of 32
 // every tile row is a full, 16-byte aligned row and moves as 16-byte copies whose
 // addresses a thread fixes once per item; otherwise element copies (a separate
 // instantiation). A thread keeps u of its own cells at z - 1, z and z + 1 in three

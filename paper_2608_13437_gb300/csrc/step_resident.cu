@@ -2,7 +2,7 @@
 //
 // A grid of up to about 58 thousand cells (one brick of at most 384 cells per SM) is far
 // too small to be bound by memory: a step moves its 98 populations per cell through the
-// L2 for no reason but that launches end, and costs 3.1 us at 16 thousand cells, of which
+// L2 for no reason but that launches end, and costs 3.3 us at 16 thousand cells, of which
 // about 1 us is the gap between two launches and most of the rest one chain of dependent
 // loads, arithmetic and stores. Here each block keeps a brick of cells for n steps, one
 // thread per cell with its 14 x 7 populations in registers (255 of them for bricks of up to
@@ -487,8 +487,9 @@ bool resident_plan(const DomainConst& P, int store, int sms, ResidentPlan* R, lo
   }
   // Against the plain kernel's nanoseconds at these sizes, fitted to the same domains (FP32);
   // with 16-bit storage the plain kernel was slower on all of them. Resident against plain,
-  // FP32: 1.6 us at 1024 x 4 x 4 (3.1), 2.95 at 32^3 (3.8), 4.1 at 38^3 (5.5), 1.95 at 16^3
-  // (2.2), 2.05 at 20 x 12 x 9 (2.2); FP16 1.6 (2.8), 2.6 (3.1), 3.8 (4.6), 2.0 (2.6).
+  // 1000 steps a call, FP32: 1.66 us at 1024 x 4 x 4 (3.28), 3.28 at 32^3 (4.17), 3.95 at 38^3
+  // (5.40), 2.05 at 24^3 (3.02), 2.30 at 20 x 12 x 9 (2.45); FP16 1.66 (3.48), 2.88 (3.66),
+  // 3.67 (4.43), 2.02 (3.22), 2.30 (2.89) and 2.20 at 16^3 (3.02).
   if (best < 0) return false;
   *plan_cost = best;
   return store != 0 || best < plain_cost(P, store, 1);
