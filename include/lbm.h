@@ -255,12 +255,14 @@ lbm_status lbm_init_state(lbm_handle* h, const void* Q, int src_on_device, int d
  * sensor and collision in FP32 and writes the 98 post-collision populations back
  * in place, so that streaming happens through the index maps. With use_graphs, calls of
  * 8 steps or more on small domains (up to about 58 thousand cells, where it is the faster
- * form) run as cooperative launches of up to 512 steps that keep the populations on the chip
+ * form) run as cooperative launches of up to 4096 steps that keep the populations on the chip
  * between the steps; the result is the same bit for bit, and a wait between its blocks that
  * runs out (bounded; it does not happen in normal operation) is reported as LBM_E_TIMEOUT.
- * Such a launch holds its SMs for 1 to 2 ms, and other kernels run beside it on the rest
- * of them; where handles with small domains live on so many streams of a device that their
- * launches would have to take turns, lbm_step launches step by step instead.
+ * Such launches hold the SMs that they use until the call's steps are done, and kernels of
+ * other streams run beside them on the rest (24 of 152 SMs beside a 32^3 domain). Where
+ * handles with small domains live on so many streams of a device that their launches would
+ * have to take turns, lbm_step launches step by step instead; so it does with use_graphs = 0
+ * or after lbm_set_kernel_config.
  * Asynchronous on the handle's stream. Returns LBM_E_STATE before
  * an init, LBM_E_NONFINITE if an earlier synchronising call saw non-finite
  * moments (no work is issued then). */

@@ -212,10 +212,12 @@ namespace {
 
 constexpr int kChunkPairs = 16;  // a chunk graph holds 32 steps
 // The resident form is taken for calls of at least this many steps (a launch loads and
-// stores the whole state once); one launch of it takes at most kResidentMostSteps, 1 to 2 ms,
-// after which kernels that wait for its SMs on other streams get their turn.
+// stores the whole state once); one launch of it takes at most kResidentMostSteps. Shorter
+// launches give other streams nothing: the next one takes the SMs back at once (two 256^3
+// steps behind 2000 steps of a 32^3 on another stream are done after 8.4 ms with launches
+// of 4096 steps and of 512; each launch costs about 8 us).
 constexpr int kResidentLeastSteps = 8;
-constexpr int kResidentMostSteps = 512;
+constexpr int kResidentMostSteps = 4096;
 
 // The streams of the live handles with a resident plan. Launches on different streams would
 // compete for the SMs, so lbm_step weighs their number (resident_pays); results do not
