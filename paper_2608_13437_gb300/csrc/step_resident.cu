@@ -179,6 +179,10 @@ __global__ void __launch_bounds__(MAXT, 1)
   constexpr int NW = Words<S>::n, NP = Words<S>::packets;
   extern __shared__ __align__(16) unsigned char smem[];
   const int steps = run.steps;
+  const unsigned epoch = epochs[blockIdx.x];
+  // Nothing is done with the incomplete state that a launch before this one left, nor by a
+  // block that is to fail: its neighbours wait in vain. (Both loads run beside the set-up.)
+  const bool idle = threadIdx.x == 0 && (gave_up(flag) || (int)blockIdx.x == run.silent);
   const int T = blockDim.x, tid = threadIdx.x;
   // exchange buffers (one, or two for even and odd tags), the rest populations of the last
   // step, and the table of the packet sets that arrive from outside
@@ -245,10 +249,7 @@ __global__ void __launch_bounds__(MAXT, 1)
       n_in += 2 * w[u] * w[v];
     }
   }
-  const unsigned epoch = epochs[blockIdx.x];
-  // Nothing is done with the incomplete state that a launch before this one left, nor by a
-  // block that is to fail: its neighbours wait in vain.
-  if (__syncthreads_or(tid == 0 && (gave_up(flag) || (int)blockIdx.x == run.silent))) {
+  if (__syncthreads_or(idle)) {
     if (tid == 0) epochs[blockIdx.x] = epoch + (unsigned)steps;
     return;
   }
